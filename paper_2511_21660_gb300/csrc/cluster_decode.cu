@@ -164,7 +164,6 @@ __global__ void __launch_bounds__(NT, VPT <= 8 && DC <= 16 ? 2 : 1) cluster_deco
     uint32_t *fb = fw + g.f_words;
     uint32_t *sg = fb + g.f_words;
     uint32_t *par = sg + 2 * g.syn_words;
-    float *ws = reinterpret_cast<float *>(par + 2 * g.m_words);
     __shared__ int s_shot, s_ns, s_ne, s_status, s_c, s_head, s_count, s_steps, s_nint, s_valid;
     __shared__ uint32_t s_x[32];
     // the shots: list[0 .. counter[1]) (the host's compaction of a skip mask), else 0 .. B-1
@@ -191,7 +190,7 @@ __global__ void __launch_bounds__(NT, VPT <= 8 && DC <= 16 ? 2 : 1) cluster_deco
             s_steps = 0;
         }
         plain_bp<NT, VPT, DC, DV>(g, p, a.bp_iters, syn + (size_t)shot * g.syn_words, msg, fw,
-                                  sg, par, ws, Lam, bb, gg);
+                                  sg, par, Lam, bb, gg);
 
         // 2. partial correction and erasures; sigma + H F_pre
         uint32_t pmask = 0u;

@@ -17,7 +17,7 @@ namespace {
 
 // Marginals of plain BP after `iters` iterations into Lam (fault threadIdx.x + r NT in
 // Lam[r]).  Shared memory: the float32 message slots (msg), the staged syndrome (sg) and
-// one parity buffer (par, zeroed by each check pass and otherwise unused).  Re-stages the
+// one parity buffer (par, set by each check pass and otherwise unused).  Re-stages the
 // padding slots first (callers reuse the message area between shots).  Called by every
 // thread of the block; ends with a barrier.
 template <int NT, int VPT, int DC, int DV>
@@ -31,6 +31,10 @@ __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C,
         for (int k = deg; k < DC; ++k) Msg<float>::st(msg, (i * DC + (k ^ f)) * 4, C);
     }
     load_syndrome<NT>(g, sy, sg);
+    const int packed = packed_slots<float, NT, VPT, DV>(g);
+    RowBits rb;
+    rb.part = partial_rows<float, NT, DC>(g);
+    const uint2 *rec = Packed<float, NT * VPT>::table(g) + threadIdx.x;
     // nu(0) = lambda(0) = w on every edge, Lambda(0) = w
     float wr[VPT];
 #pragma unroll
@@ -48,19 +52,24 @@ __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C,
                 if (k < deg) Msg<float>::st(msg, sl[k], w);
         }
     }
+    row_syndromes<float, NT>(g, sy, rb);
     __syncthreads();
     for (int t = 0; t < iters; ++t) {
-        check_pass<NT, DC>(g, reinterpret_cast<float *>(msg), sg, par, C);
+        check_pass<NT, DC>(g, reinterpret_cast<float *>(msg), sg, par, rb, C);
         __syncthreads();
-#pragma unroll
-        for (int r = 0; r < VPT; ++r) {
+        auto fast = [&](int r) {
+            const Packed<float, NT * VPT> s(__ldg(rec + r * NT));
+            Lam[r] = fault_update(msg, s, wr[r], C);
+        };
+        auto any = [&](int r) {
             const int j = threadIdx.x + r * NT;
             if (j < g.N) {
                 int sl[DV];
                 const int deg = load_slots<DV>(g, j, sl);
                 Lam[r] = fault_update<float, DV>(msg, sl, deg, wr[r], C);
             }
-        }
+        };
+        each_fault<VPT>(packed, fast, any);
         __syncthreads();
     }
 }

@@ -121,7 +121,7 @@ __host__ __device__ inline size_t cluster_union_bytes(const FusedGraph &g, const
 }
 inline size_t cluster_smem_bytes(const FusedGraph &g, const ClusterArgs &a) {
     return cluster_union_bytes(g, a) + 8 * (size_t)g.f_words + 8 * (size_t)g.syn_words +
-           8 * (size_t)g.m_words + 4 * (size_t)g.N + 64;
+           8 * (size_t)g.m_words + 64;
 }
 
 }  // namespace qldpc

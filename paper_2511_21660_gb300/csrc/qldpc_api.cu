@@ -192,6 +192,13 @@ void place_edges(int M, int N, int DV, const int32_t *row_ptr, const int32_t *co
     }
 }
 
+// Whether a compiled shape holds a graph: its fault slots, and the 32 check rows a thread
+// keeps bits for (rows of check pairs with binary16 messages).
+bool holds(const FusedKernel &k, int M, int N) {
+    const long long rows = k.msg_fp16 ? (M + 1) / 2 : M;
+    return (long long)k.threads * k.vpt >= N && 32LL * k.threads >= rows;
+}
+
 // Tail continuation: the resuming launch runs the compiled 1024-thread shape with the
 // fewest faults per thread that holds N (one block per SM; none holds it: no
 // continuation); 4 records per SM.  tail_cut < 0 turns it off, 0 picks T_1 + 8 T_r.
@@ -234,7 +241,7 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     if (rc) return rc;
     const int DC = tab[0].dc, DV = tab[0].dv;
     for (int q = 0; q < ntab && !d->fk; ++q)
-        if ((long long)tab[q].threads * tab[q].vpt >= N &&
+        if (holds(tab[q], M, N) &&
             (block_threads == 0 || tab[q].threads == block_threads))
             d->fk = &tab[q];
     if (!d->fk)
@@ -251,6 +258,8 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     g.cor_words = (N + 63) / 64;
     g.f_words = (2 * g.cor_words + 2 + 3) & ~3;  // whole 16-byte groups
     g.m_words = (M + 31) / 32;
+    g.min_deg = DC;
+    for (int i = 0; i < M; ++i) g.min_deg = std::min(g.min_deg, row_ptr[i + 1] - row_ptr[i]);
 
     // message layout (see FusedGraph): rows of DC slots, swizzled inside a row
     const bool half = d->msg_fp16 != 0;
@@ -283,20 +292,38 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
             var_slot[(size_t)j * DV + var_deg[j]++] = off;  // rows ascending => checks ascending
         }
     }
-    for (int j = 0; j < N; ++j) var_slot[(size_t)j * DV] |= var_deg[j] << 24;
+    // packed slot records: [0, N) in messages, [N, 2 N) in bytes
+    const bool rec_fits = g.msg_bytes / msg_size <= 65536, rec8_fits = g.msg_bytes <= 65536;
+    std::vector<uint32_t> var_rec(4 * (size_t)N, 0u);
+    for (int j = 0; j < N; ++j) {
+        const int32_t *sl = &var_slot[(size_t)j * DV];
+        if (var_deg[j] == 2 || var_deg[j] == 3)
+            for (int u = 0; u < 2; ++u) {
+                const uint32_t unit = u ? 1u : (uint32_t)msg_size;
+                const uint32_t s0 = sl[0] / unit, s1 = sl[1] / unit;
+                const uint32_t s2 = var_deg[j] == 3 ? sl[2] / unit : s0;
+                uint32_t *r = &var_rec[2 * ((size_t)u * N + j)];
+                if (u ? !rec8_fits : !rec_fits) continue;
+                r[0] = s0 | (s1 << 16);
+                r[1] = s2 | ((uint32_t)var_deg[j] << 16);
+            }
+        var_slot[(size_t)j * DV] |= var_deg[j] << 24;
+    }
     for (int i = 0; i < g.Mp; ++i)
         for (int k = chk_deg[i]; k < DC; ++k) {
             const int p = k ^ swz(i >> 1);
             pad_mask[(size_t)(i / 2) * DC + p] |= (i & 1) ? 0xffff0000u : 0x0000ffffu;
         }
 
-    d->smem = fused_smem_bytes(g.msg_bytes, g.f_words, g.syn_words, g.m_words, N);
+    d->smem = fused_smem_bytes(g.msg_bytes, g.f_words, g.syn_words, g.m_words);
     int optin = 0;
     QL_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, d->device));
     QL_CUDA(cudaDeviceGetAttribute(&d->num_sms, cudaDevAttrMultiProcessorCount, d->device));
-    if (d->smem > (size_t)optin)
+    // the size limit of the entry point: the kernels' state and 4 bytes a fault
+    const size_t state = d->smem + sizeof(float) * N;
+    if (state > (size_t)optin)
         return fail(QLDPC_ERR_UNSUPPORTED, "per-shot state needs %zu B of shared memory, above %d",
-                    d->smem, optin);
+                    state, optin);
     QL_CUDA(cudaFuncSetAttribute(d->fk->decode_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)d->smem));
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->blocks_per_sm, d->fk->decode_fn,
@@ -313,19 +340,20 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
 
     // one device arena for every graph array
     const size_t R1 = (size_t)d->prm.R + 1;
-    size_t off[8], o = 0;
-    const size_t sizes[8] = {(size_t)g.Mp, sizeof(int32_t) * N * DV, sizeof(uint32_t) * pad_mask.size(),
+    size_t off[9], o = 0;
+    const size_t sizes[9] = {(size_t)g.Mp, sizeof(int32_t) * N * DV, sizeof(uint32_t) * pad_mask.size(),
                              sizeof(int32_t) * N * DV, sizeof(float) * N, sizeof(float) * R1 * N,
-                             sizeof(int32_t) * slot_edge.size(), sizeof(unsigned int) * 4};
-    for (int q = 0; q < 8; ++q) {
+                             sizeof(int32_t) * slot_edge.size(), sizeof(uint32_t) * var_rec.size(),
+                             sizeof(unsigned int) * 4};
+    for (int q = 0; q < 9; ++q) {
         off[q] = o;
         o = align_up(o + sizes[q], 256);
     }
     QL_CUDA(cudaMalloc(&d->arena, o));
     char *base = static_cast<char *>(d->arena);
-    const void *src[7] = {chk_deg.data(), var_chk.data(), pad_mask.data(), var_slot.data(),
-                          w.data(), gamma, slot_edge.data()};
-    for (int q = 0; q < 7; ++q)
+    const void *src[8] = {chk_deg.data(), var_chk.data(), pad_mask.data(), var_slot.data(),
+                          w.data(), gamma, slot_edge.data(), var_rec.data()};
+    for (int q = 0; q < 8; ++q)
         QL_CUDA(cudaMemcpy(base + off[q], src[q], sizes[q], cudaMemcpyHostToDevice));
     g.chk_deg = reinterpret_cast<const uint8_t *>(base + off[0]);
     g.var_chk = reinterpret_cast<const int32_t *>(base + off[1]);
@@ -334,7 +362,10 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     g.w = reinterpret_cast<const float *>(base + off[4]);
     g.gamma = reinterpret_cast<const float *>(base + off[5]);
     g.slot_edge = reinterpret_cast<const int32_t *>(base + off[6]);
-    d->counter = reinterpret_cast<unsigned int *>(base + off[7]);
+    const uint2 *rec = reinterpret_cast<const uint2 *>(base + off[7]);
+    g.var_rec = rec_fits ? rec : nullptr;
+    g.var_rec8 = rec8_fits ? rec + N : nullptr;
+    d->counter = reinterpret_cast<unsigned int *>(base + off[8]);
     QL_CUDA(cudaMemset(d->counter, 0, sizeof(unsigned int) * 4));
     return setup_tail(d, tab, ntab, tail_cut);
 }

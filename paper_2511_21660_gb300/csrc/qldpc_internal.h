@@ -33,10 +33,15 @@ struct FusedGraph {
     int f_words;          // uint32 words of the decision bitmap (2*cor_words + 2, rounded
                           // up to a multiple of 4)
     int m_words;          // ceil(M/32) uint32 words of a parity bitmap
+    int min_deg;          // smallest check degree
     const uint8_t *chk_deg;   // [Mp] check degrees (0 for rows M..Mp-1)
     const int32_t *var_chk;   // [N][DV] checks of fault j, increasing order
     const int32_t *var_slot;  // [N][DV] byte offsets of the messages of fault j's edges,
                               // increasing check order; top byte of entry 0 = degree
+    const uint2 *var_rec;     // [N] faults of degree 2 and 3: the slots in 16-bit fields (in
+                              // messages; x = s0 | s1 << 16, y = s2 | degree << 16, degree 2
+                              // with s2 = s0); nullptr when a slot does not fit 16 bits
+    const uint2 *var_rec8;    // [N] the same with byte offsets; nullptr above 64 KB of messages
     const uint32_t *pad_mask; // [Mp/2][DC] binary16 only: 0xffff in each half of the
                               // pair's physical word p that holds a padding slot
     const float *w;           // [N] prior LLRs
@@ -133,10 +138,9 @@ struct FusedKernel {
 };
 
 // Shared memory of the fused kernels for a graph (bytes).
-inline size_t fused_smem_bytes(int msg_bytes, int f_words, int syn_words, int m_words, int N) {
+inline size_t fused_smem_bytes(int msg_bytes, int f_words, int syn_words, int m_words) {
     size_t msg = ((size_t)msg_bytes + 15) & ~(size_t)15;
-    return msg + 8 * (size_t)f_words + 8 * (size_t)syn_words + 8 * (size_t)m_words +
-           4 * (size_t)N + 64;
+    return msg + 8 * (size_t)f_words + 8 * (size_t)syn_words + 8 * (size_t)m_words + 64;
 }
 
 // Tables of compiled fused kernels, one per (precision, DC, DV) translation unit.

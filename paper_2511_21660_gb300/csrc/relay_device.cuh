@@ -37,17 +37,12 @@ struct Msg<__half> {
 
 __device__ __forceinline__ float clampc(float x, float c) { return fminf(fmaxf(x, -c), c); }
 
-// Binary16 store with saturation at the largest finite value, 65504: for every finite x
-// it equals rounding min(max(x, -65504), 65504) to nearest, i.e. the clamp to C = 65504
-// followed by the store.
-__device__ __forceinline__ void st_half_sat(unsigned char *base, int off, float v) {
-    unsigned short h;
-    asm("cvt.rn.satfinite.f16.f32 %0, %1;" : "=h"(h) : "f"(v));
-    *reinterpret_cast<unsigned short *>(base + off) = h;
-}
-
-__device__ __forceinline__ unsigned short ld_half_bits(const unsigned char *base, int off) {
-    return *reinterpret_cast<const unsigned short *>(base + off);
+// The clamp that keeps a NaN (clampc turns it into -c).
+__device__ __forceinline__ float clamp_nan(float x, float c) {
+    float y;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(x), "f"(-c));
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(y), "f"(c));
+    return y;
 }
 
 // x + h for a binary16 operand h in one float32 addition (the widening of h is exact,
@@ -56,6 +51,24 @@ __device__ __forceinline__ float add_f16(float x, unsigned short h) {
     float d;
     asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(h), "f"(x));
     return d;
+}
+
+// Messages as the fault pass takes them: the stored value as it is, added to a float32 sum.
+template <typename MT>
+struct Raw;
+template <>
+struct Raw<float> {
+    using T = float;
+    static __device__ __forceinline__ float add(float x, float m) { return __fadd_rn(x, m); }
+};
+template <>
+struct Raw<__half> {
+    using T = unsigned short;
+    static __device__ __forceinline__ float add(float x, unsigned short m) { return add_f16(x, m); }
+};
+template <typename MT>
+__device__ __forceinline__ typename Raw<MT>::T ld_raw(const unsigned char *msg, uint32_t off) {
+    return *reinterpret_cast<const typename Raw<MT>::T *>(msg + off);
 }
 
 // x + 0 = x for x != 0 and -0 + 0 = +0.  Applied to lambda(0) and to
@@ -112,97 +125,241 @@ __device__ __forceinline__ int swz(int i) {
     return (i >> sh) & (DC - 1);
 }
 
+// Packed slot records of the faults of degree 2 and 3 (8 bytes a fault: x = s0 | s1 << 16,
+// y = s2 | degree << 16; degree 2: s2 = s0).  Blocks of up to 3072 faults read byte offsets
+// (their message arrays rarely pass 64 KB); the larger shapes read offsets in messages.
+// The records are read in every fault pass: at 8 bytes the two-gross code's 64 KB stay in L1
+// beside its messages, where the 16-byte table of offsets hit in half the reads.
+template <typename MT, int FAULTS>
+struct Packed {
+    static constexpr bool kBytes = FAULTS <= 3072;
+    static __device__ __forceinline__ const uint2 *table(const FusedGraph &g) {
+        return kBytes ? g.var_rec8 : g.var_rec;
+    }
+    uint32_t o0, o1, o2;  // byte offsets of the fault's slots
+    bool three;
+    __device__ __forceinline__ explicit Packed(const uint2 q) {
+        constexpr uint32_t unit = kBytes ? 1u : (uint32_t)sizeof(MT);
+        o0 = (q.x & 0xffffu) * unit;
+        o1 = (q.x >> 16) * unit;
+        o2 = (q.y & 0xffffu) * unit;
+        three = q.y >= (3u << 16);
+    }
+};
+
+// Fault slots of the warp (faults threadIdx.x + r NT) that take the packed-record path: the
+// slots r < n, n the number of leading slots whose 32 faults all exist and have degree 2 or 3.
+// Called by whole warps.
+template <typename MT, int NT, int VPT, int DV>
+__device__ __forceinline__ int packed_slots(const FusedGraph &g) {
+    if (!Packed<MT, NT * VPT>::table(g)) return 0;
+    int r = 0;
+#pragma unroll 1
+    for (; r < VPT; ++r) {
+        const int j = threadIdx.x + r * NT;
+        int deg = 0;
+        if (j < g.N) deg = (int)((uint32_t)__ldg(g.var_slot + (size_t)j * DV) >> 24);
+        if (!__all_sync(FULL, deg == 2 || deg == 3)) break;
+    }
+    return r;
+}
+
+// The per-fault loops: fast(r) for the packed slots and any(r) for the others.  (One loop body
+// with a branch per fault on its degree, a ballot and a bitmap store took 50 instructions a
+// warp of faults, this form 31; gross code, 30,000 shots: 2.50 -> 1.96 ms with the leg
+// start's same change.)  The shapes
+// are chosen so that a graph fills every fault slot but the last, and then the loop runs
+// without a branch between faults, which lets their loads overlap; on other graphs it
+// branches once per group of faults (and takes any(r) in the group where the packed slots end).
+template <int VPT, typename Fast, typename Any>
+__device__ __forceinline__ void each_fault(int packed, Fast fast, Any any) {
+    if (packed >= VPT - 1) {
+#pragma unroll
+        for (int r = 0; r < VPT - 1; ++r) fast(r);
+        if (packed == VPT)
+            fast(VPT - 1);
+        else
+            any(VPT - 1);
+    } else {
+        constexpr int G = 4;
+#pragma unroll
+        for (int r0 = 0; r0 < VPT; r0 += G) {
+            const int r1 = r0 + G < VPT ? r0 + G : VPT;
+            if (packed >= r1) {
+#pragma unroll
+                for (int r = r0; r < r1; ++r) fast(r);
+            } else {
+#pragma unroll
+                for (int r = r0; r < r1; ++r) any(r);
+            }
+        }
+    }
+}
+
 // Start of a leg: lambda(0), Lambda(0), nu(0) and the leg's memory strengths.
 //   leg 0:  lambda(0) = Lambda(0) = w
 //   leg r:  Lambda(0) = previous terminal marginals; lambda(0) = Lambda(0)
 //           (warm_mode 0) or w (warm_mode 1); nu(0) = lambda(0)
 // bb holds (1 - gamma_j) * lambda_j(0), rounded, which is the first product of
 // the memory update and is constant within a leg.
-template <typename MT, int NT, int VPT, int DV, bool SKIP = false>
+template <typename MT, int NT, int VPT, int DV>
 __device__ __forceinline__ void leg_init(const FusedGraph &g, const DevParams &p, int leg,
-                                         unsigned char *msg, const float *ws, float (&Lam)[VPT],
-                                         float (&bb)[VPT], float (&gg)[VPT]) {
-    const float *grow = g.gamma + (size_t)leg * g.N;
+                                         unsigned char *msg, int packed,
+                                         float (&Lam)[VPT], float (&bb)[VPT],
+                                         float (&gg)[VPT]) {
+    const float *grow = g.gamma + (size_t)leg * g.N + threadIdx.x;
+    const uint2 *rec = Packed<MT, NT * VPT>::table(g) + threadIdx.x;
+    if (leg == 0 || p.warm_mode == 1) {  // lambda(0) = w
 #pragma unroll
-    for (int r = 0; r < VPT; ++r) {
-        if (SKIP && r * NT >= g.N) break;  // the block's remaining fault slots are empty
+        for (int r = 0; r < VPT; ++r) {
+            const int j = threadIdx.x + r * NT;
+            if (j < g.N) bb[r] = canon(__ldg(g.w + j));
+        }
+        if (leg == 0) {
+#pragma unroll
+            for (int r = 0; r < VPT; ++r) Lam[r] = bb[r];
+        }
+    } else {  // lambda(0) = Lambda
+#pragma unroll
+        for (int r = 0; r < VPT; ++r) bb[r] = canon(Lam[r]);
+    }
+    auto fast = [&](int r) {
+        const Packed<MT, NT * VPT> s(__ldg(rec + r * NT));
+        const float lam0 = bb[r], gm = __ldg(grow + r * NT);
+        Msg<MT>::st(msg, s.o0, lam0);
+        Msg<MT>::st(msg, s.o1, lam0);
+        if (s.three) Msg<MT>::st(msg, s.o2, lam0);
+        gg[r] = gm;
+        bb[r] = canon(__fmul_rn(__fsub_rn(1.0f, gm), lam0));
+    };
+    auto any = [&](int r) {
         const int j = threadIdx.x + r * NT;
         if (j < g.N) {
-            const float lam0 = canon((leg == 0 || p.warm_mode == 1) ? ws[j] : Lam[r]);
-            if (leg == 0) Lam[r] = lam0;
-            const float gm = __ldg(grow + j);
-            gg[r] = gm;
-            bb[r] = canon(__fmul_rn(__fsub_rn(1.0f, gm), lam0));
+            const float lam0 = bb[r], gm = __ldg(grow + r * NT);
             int sl[DV];
             const int deg = load_slots<DV>(g, j, sl);
 #pragma unroll
             for (int k = 0; k < DV; ++k)
                 if (k < deg) Msg<MT>::st(msg, sl[k], lam0);
+            gg[r] = gm;
+            bb[r] = canon(__fmul_rn(__fsub_rn(1.0f, gm), lam0));
+        }
+    };
+    each_fault<VPT>(packed, fast, any);
+}
+
+// The check rule's combination of two messages: the smaller magnitude with the product of
+// the signs, in one instruction (per half for a pair of binary16 values).  Exact and
+// independent of the order of combination.  min, max, compare, select and logic all issue on
+// the half-rate ALU pipe, which the check pass is bound by: the two smallest magnitudes, a
+// select per slot and separate sign logic took 41 ALU instructions a warp of rows, this form
+// 26 (gross code, 30,000 shots at p = 0.003, 384 threads: 1.96 -> 1.77 ms).
+__device__ __forceinline__ float minsign(float a, float b) {
+    float d;
+    asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ uint32_t minsign(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("min.xorsign.abs.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// o_k = the combination of rest and every a_l, l != k: pairs are combined on the way up, and
+// on the way down each element meets its sibling and what lies outside the pair
+// (n = 8: 20 combinations).
+template <int n, typename V>
+__device__ __forceinline__ void excluded(const V (&a)[n], V rest, V (&o)[n]) {
+    static_assert(n >= 2 && (n & (n - 1)) == 0, "power-of-two row capacity");
+    if constexpr (n == 2) {
+        o[0] = minsign(a[1], rest);
+        o[1] = minsign(a[0], rest);
+    } else {
+        V p[n / 2], e[n / 2];
+#pragma unroll
+        for (int k = 0; k < n / 2; ++k) p[k] = minsign(a[2 * k], a[2 * k + 1]);
+        excluded<n / 2>(p, rest, e);
+#pragma unroll
+        for (int k = 0; k < n / 2; ++k) {
+            o[2 * k] = minsign(a[2 * k + 1], e[k]);
+            o[2 * k + 1] = minsign(a[2 * k], e[k]);
         }
     }
 }
 
-// Two smallest of n values (with multiplicity) by a pairwise tree: sorted pairs, then
-// merges of sorted pairs, (l, h) = (min(l1, l2), min(max(l1, l2), min(h1, h2))).  min
-// and max are exact, so the result is the one a sequential scan gives, in log2(n)
-// dependent steps instead of n.  V is float or __half2 (two checks at once).
-__device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ __half2 vmin(__half2 a, __half2 b) { return __hmin2(a, b); }
-__device__ __forceinline__ __half2 vmax(__half2 a, __half2 b) { return __hmax2(a, b); }
+// What a thread keeps for its check rows (row k of the thread: threadIdx.x + k NT; rows of
+// check pairs with binary16 messages): bit k of s0 (and of s1 for the pair's second check)
+// is the syndrome bit, bit k of part says that the row has padding slots.
+struct RowBits {
+    uint32_t s0, s1, part;
+};
 
-// Rows wider than 8 slots keep the sequential scan (the tree's live values would spill).
-template <int n, typename V>
-__device__ __forceinline__ void two_smallest(const V (&a)[n], V &m1, V &m2) {
-    static_assert(n >= 2 && (n & (n - 1)) == 0, "power-of-two row capacity");
-    if constexpr (n > 8) {
-        m1 = vmin(a[0], a[1]);
-        m2 = vmax(a[0], a[1]);
-#pragma unroll
-        for (int k = 2; k < n; ++k) {
-            m2 = vmin(m2, vmax(m1, a[k]));
-            m1 = vmin(m1, a[k]);
+template <typename MT, int NT, int DC>
+__device__ __forceinline__ uint32_t partial_rows(const FusedGraph &g) {
+    uint32_t m = 0u;
+    const bool half = sizeof(MT) == 2;
+    const int rows = half ? (g.M + 1) >> 1 : g.M;
+    for (int i = threadIdx.x, k = 0; i < rows; i += NT, ++k) {
+        const bool full = half ? g.chk_deg[2 * i] == DC && g.chk_deg[2 * i + 1] == DC
+                               : g.chk_deg[i] == DC;
+        m |= (full ? 0u : 1u) << k;
+    }
+    return m;
+}
+
+// The syndrome bits of the thread's rows, from the shot's packed words in global memory.
+template <typename MT, int NT>
+__device__ __forceinline__ void row_syndromes(const FusedGraph &g, const uint64_t *sy,
+                                              RowBits &rb) {
+    rb.s0 = rb.s1 = 0u;
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(sy);
+    const bool half = sizeof(MT) == 2;
+    const int rows = half ? (g.M + 1) >> 1 : g.M;
+#pragma unroll 1
+    for (int i = threadIdx.x, k = 0; i < rows; i += NT, ++k) {
+        if (half) {
+            const uint32_t b = __ldg(w + (i >> 4)) >> (2 * (i & 15));
+            rb.s0 |= (b & 1u) << k;
+            rb.s1 |= ((b >> 1) & 1u) << k;
+        } else {
+            rb.s0 |= ((__ldg(w + (i >> 5)) >> (i & 31)) & 1u) << k;
         }
-        return;
     }
-    V lo[n / 2], hi[n / 2];
-#pragma unroll
-    for (int k = 0; k < n / 2; ++k) {
-        lo[k] = vmin(a[2 * k], a[2 * k + 1]);
-        hi[k] = vmax(a[2 * k], a[2 * k + 1]);
-    }
-#pragma unroll
-    for (int w = n / 2; w > 1; w >>= 1) {
-#pragma unroll
-        for (int k = 0; k < w / 2; ++k) {
-            const V l = vmin(lo[2 * k], lo[2 * k + 1]);
-            hi[k] = vmin(vmax(lo[2 * k], lo[2 * k + 1]), vmin(hi[2 * k], hi[2 * k + 1]));
-            lo[k] = l;
-        }
-    }
-    m1 = lo[0];
-    m2 = hi[0];
+}
+
+// The parity words start an iteration as the syndrome.
+template <int NT>
+__device__ __forceinline__ void set_parity(const FusedGraph &g, const uint32_t *sg,
+                                           uint32_t *par) {
+    if (threadIdx.x >= g.m_words) return;
+    par[threadIdx.x] = sg[threadIdx.x];
+    for (int q = threadIdx.x + NT; q < g.m_words; q += NT) par[q] = sg[q];
 }
 
 // Check pass, float32 messages: mu_{i->j}(t) from nu(t-1) for every check, in place.
-// (m1, m2) = the two smallest magnitudes of the check's slots (with multiplicity) and
-// of {C, C}, so the min over the excluded set of slot k is m2 if |nu_k| = m1, else m1.
-// Padding slots hold C, which is also the min over an empty set, and keep it.
-// The sign is (-1)^sigma_i times the product of all signs times sign(nu_k).
+// Slot k gets the combination of every other slot of the row and of (-1)^sigma_i C: the
+// smallest other magnitude, at most C, with the product of the other signs and the check's.
+// The minimum with C also stands for the clamp of nu to [-C, C]: min(|nu|, C) is the clamped
+// magnitude and a clamp keeps the sign, so the fault pass stores nu unclamped.
+// Padding slots hold +C, the neutral value here, and keep it.
 // Slots are processed in physical order: the rule does not depend on the order.
 // Lanes read and write their row's 16-byte chunks in the order k4 ^ cs: rows are
 // 4*DC bytes apart, and cs = (row / rows per 128-byte line) mod chunks per row makes
 // each 128-bit access of a warp touch every bank equally often (no bank conflict).
+// NT is a multiple of 32, so cs and the swizzle are the same for all rows of a thread.
+// The parity words start the iteration as the syndrome (the fault pass flips them to 0).
 template <int NT, int DC>
 __device__ __forceinline__ void check_pass(const FusedGraph &g, float *msg, const uint32_t *sg,
-                                           uint32_t *par_zero, float C) {
-    for (int q = threadIdx.x; q < g.m_words; q += NT) par_zero[q] = 0u;
+                                           uint32_t *par, const RowBits &rb, float C) {
+    set_parity<NT>(g, sg, par);
+    static_assert(NT % 32 == 0, "the chunk order and the swizzle repeat every 32 rows");
+    const int cs = (threadIdx.x / (DC >= 32 ? 1 : 32 / DC)) & (DC / 4 - 1);  // chunk order
+    const uint32_t c = __float_as_uint(C);
+    float4 *row = reinterpret_cast<float4 *>(msg + (size_t)threadIdx.x * DC);
+    uint32_t sb = rb.s0, part = rb.part;
+#pragma unroll 1
     for (int i = threadIdx.x; i < g.M; i += NT) {
-        const int deg = g.chk_deg[i];
-        uint32_t sx = sg[i >> 5] << (31 - (i & 31));
-        float4 *row = reinterpret_cast<float4 *>(msg + (size_t)i * DC);
-        const int cs = (i / (DC >= 32 ? 1 : 32 / DC)) & (DC / 4 - 1);  // chunk order
-        float v[DC];
+        float v[DC], o[DC];
 #pragma unroll
         for (int k4 = 0; k4 < DC / 4; ++k4) {
             const float4 t = row[k4 ^ cs];
@@ -211,62 +368,40 @@ __device__ __forceinline__ void check_pass(const FusedGraph &g, float *msg, cons
             v[4 * k4 + 2] = t.z;
             v[4 * k4 + 3] = t.w;
         }
-        float a[DC], m1, m2;
-        uint32_t x[DC / 2];
-#pragma unroll
-        for (int k = 0; k < DC; ++k) a[k] = fabsf(v[k]);
-        two_smallest<DC>(a, m1, m2);
-        m1 = fminf(m1, C);
-        m2 = fminf(m2, C);
-#pragma unroll
-        for (int k = 0; k < DC / 2; ++k)
-            x[k] = __float_as_uint(v[2 * k]) ^ __float_as_uint(v[2 * k + 1]);
-#pragma unroll
-        for (int w = DC / 2; w > 1; w >>= 1)
-#pragma unroll
-            for (int k = 0; k < w / 2; ++k) x[k] = x[2 * k] ^ x[2 * k + 1];
-        sx = (sx ^ x[0]) & 0x80000000u;
-        // Slot k holds a smallest magnitude iff |nu_k| <= m1 (no |nu_k| is below m1);
-        // its excluded minimum is then m2 (= m1 on a tie), else m1.  Both candidates
-        // carry the sign of the whole product; one XOR takes the slot's own sign out.
-        const uint32_t s1 = __float_as_uint(m1) | sx, s2 = __float_as_uint(m2) | sx;
-        float o[DC];
-#pragma unroll
-        for (int k = 0; k < DC; ++k) {
-            const uint32_t c = a[k] <= m1 ? s2 : s1;
-            o[k] = __uint_as_float(c ^ (__float_as_uint(v[k]) & 0x80000000u));
-        }
-        if (deg < DC) {  // v[k] is physical slot k ^ 4cs, logical slot k ^ 4cs ^ swz(i)
-            const int f = swz<DC>(i) ^ (cs << 2);
-#pragma unroll
-            for (int k = 0; k < DC; ++k)
-                if ((k ^ f) >= deg) o[k] = C;
-        }
+        excluded<DC>(v, __uint_as_float((sb << 31) | c), o);
 #pragma unroll
         for (int k4 = 0; k4 < DC / 4; ++k4)
             row[k4 ^ cs] = make_float4(o[4 * k4], o[4 * k4 + 1], o[4 * k4 + 2], o[4 * k4 + 3]);
+        if (part & 1u) {  // padding slots get C back: the last slot, seldom more
+            float *r = reinterpret_cast<float *>(row);
+            r[(DC - 1) ^ swz<DC>(threadIdx.x)] = C;
+            if (g.min_deg < DC - 1)
+                for (int k = g.chk_deg[i]; k < DC - 1; ++k) r[k ^ swz<DC>(threadIdx.x)] = C;
+        }
+        row += NT * DC / 4;
+        sb >>= 1;
+        part >>= 1;
     }
 }
 
 // Check pass, binary16 messages: checks 2q and 2q+1 share each 32-bit word (low
-// and high half), processed together with half2 arithmetic; min, max and sign
-// manipulation are exact in any format.  A per-pair mask keeps C in padding halves.
+// and high half), processed together; minima and signs are exact in any format.  A per-pair
+// mask keeps C in padding halves.
 // Row chunks are visited in the order k4 ^ cs as in the float32 pass (rows of check
 // pairs are 4*DC bytes apart too); only the padding mask follows the order.
 template <int NT, int DC>
 __device__ __forceinline__ void check_pass(const FusedGraph &g, __half *msg, const uint32_t *sg,
-                                           uint32_t *par_zero, float C) {
-    for (int q = threadIdx.x; q < g.m_words; q += NT) par_zero[q] = 0u;
+                                           uint32_t *par, const RowBits &rb, float C) {
+    set_parity<NT>(g, sg, par);
     const __half2 C2 = __float2half2_rn(C);
     const uint32_t c2 = *reinterpret_cast<const uint32_t *>(&C2);
     const int M2 = (g.M + 1) >> 1;
+    const int cs = (threadIdx.x / (DC >= 32 ? 1 : 32 / DC)) & (DC / 4 - 1);
+    uint4 *row = reinterpret_cast<uint4 *>(msg + (size_t)threadIdx.x * 2 * DC);
+    uint32_t sb0 = rb.s0, sb1 = rb.s1, part = rb.part;
+#pragma unroll 1
     for (int q = threadIdx.x; q < M2; q += NT) {
-        const int i = 2 * q;
-        const uint32_t sb = (sg[i >> 5] >> (i & 31)) & 3u;
-        uint32_t sx = ((sb & 1u) << 15) | ((sb & 2u) << 30);
-        const bool full = g.chk_deg[i] == DC && g.chk_deg[i + 1] == DC;
-        uint4 *row = reinterpret_cast<uint4 *>(msg + (size_t)q * 2 * DC);
-        const int cs = (q / (DC >= 32 ? 1 : 32 / DC)) & (DC / 4 - 1);
+        const uint32_t sx = (sb1 << 31) | ((sb0 & 1u) << 15);
         uint32_t v[DC];
 #pragma unroll
         for (int k4 = 0; k4 < DC / 4; ++k4) {
@@ -276,30 +411,9 @@ __device__ __forceinline__ void check_pass(const FusedGraph &g, __half *msg, con
             v[4 * k4 + 2] = t.z;
             v[4 * k4 + 3] = t.w;
         }
-        __half2 a[DC], m1, m2;
-        uint32_t x[DC / 2];
-#pragma unroll
-        for (int k = 0; k < DC; ++k) a[k] = __habs2(*reinterpret_cast<const __half2 *>(&v[k]));
-        two_smallest<DC>(a, m1, m2);
-        m1 = __hmin2(m1, C2);
-        m2 = __hmin2(m2, C2);
-#pragma unroll
-        for (int k = 0; k < DC / 2; ++k) x[k] = v[2 * k] ^ v[2 * k + 1];
-#pragma unroll
-        for (int w = DC / 2; w > 1; w >>= 1)
-#pragma unroll
-            for (int k = 0; k < w / 2; ++k) x[k] = x[2 * k] ^ x[2 * k + 1];
-        sx = (sx ^ x[0]) & 0x80008000u;
-        const uint32_t u1 = *reinterpret_cast<const uint32_t *>(&m1);
-        const uint32_t u2 = *reinterpret_cast<const uint32_t *>(&m2);
-        const uint32_t s1 = u1 | sx, s2 = u2 | sx;  // candidates with the product's sign
         uint32_t o[DC];
-#pragma unroll
-        for (int k = 0; k < DC; ++k) {
-            const uint32_t eq = __hle2_mask(a[k], m1);
-            o[k] = ((s2 & eq) | (s1 & ~eq)) ^ (v[k] & 0x80008000u);
-        }
-        if (!full) {
+        excluded<DC>(v, c2 | sx, o);
+        if (part & 1u) {
             const uint4 *pm4 = reinterpret_cast<const uint4 *>(g.pad_mask + (size_t)q * DC);
 #pragma unroll
             for (int k4 = 0; k4 < DC / 4; ++k4) {
@@ -313,152 +427,147 @@ __device__ __forceinline__ void check_pass(const FusedGraph &g, __half *msg, con
 #pragma unroll
         for (int k4 = 0; k4 < DC / 4; ++k4)
             row[k4 ^ cs] = make_uint4(o[4 * k4], o[4 * k4 + 1], o[4 * k4 + 2], o[4 * k4 + 3]);
+        row += NT * DC / 4;
+        sb0 >>= 1;
+        sb1 >>= 1;
+        part >>= 1;
     }
 }
 
-// Fault update for one fault: memory term, marginal, excluded sums (increasing check
-// order, one rounding per addition, exactly as written in the oracle).
+// Fault update for one fault: marginal and excluded sums (increasing check order, one
+// rounding per addition, as written in the oracle).  A slot the fault does not have adds
+// +0, which changes no sum (none is -0: they start from lambda, which canon keeps from
+// -0).  Messages are stored unclamped (the check pass takes their magnitudes' minimum
+// with C); the marginal is clamped.
+//
+// Faults of degree 2 and 3 with their slots in a packed record.
+template <typename MT, int FAULTS>
+__device__ __forceinline__ float fault_update(unsigned char *msg, const Packed<MT, FAULTS> &s,
+                                              float lam, float C) {
+    using R = Raw<MT>;
+    const typename R::T m0 = ld_raw<MT>(msg, s.o0), m1 = ld_raw<MT>(msg, s.o1);
+    typename R::T m2 = 0;
+    if (s.three) m2 = ld_raw<MT>(msg, s.o2);
+    const float p1 = R::add(lam, m0), p2 = R::add(p1, m1);
+    Msg<MT>::st(msg, s.o0, R::add(R::add(lam, m1), m2));
+    Msg<MT>::st(msg, s.o1, R::add(p1, m2));
+    if (s.three) Msg<MT>::st(msg, s.o2, p2);
+    const float L = R::add(p2, m2);
+    return sizeof(MT) == 4 ? clamp_nan(L, C) : clampc(L, C);
+}
+
+// Any degree up to DV.
 template <typename MT, int DV>
 __device__ __forceinline__ float fault_update(unsigned char *msg, const int (&sl)[DV], int deg,
                                               float lam, float C) {
-    // binary16 storage with C = 65504 (its default): the saturating store clamps the
-    // messages, so only the marginal needs an explicit clamp
-    // the binary16 operands enter the float32 sums through mixed-precision additions
-    if constexpr (sizeof(MT) == 2) {
-        if (C == 65504.0f && (deg == 3 || deg == 2)) {
-            const unsigned short mu0 = ld_half_bits(msg, sl[0]), mu1 = ld_half_bits(msg, sl[1]);
-            const float s0 = add_f16(lam, mu0);
-            if (deg == 3) {
-                const unsigned short mu2 = ld_half_bits(msg, sl[2]);
-                const float s01 = add_f16(s0, mu1);
-                st_half_sat(msg, sl[0], add_f16(add_f16(lam, mu1), mu2));
-                st_half_sat(msg, sl[1], add_f16(s0, mu2));
-                st_half_sat(msg, sl[2], s01);
-                return clampc(add_f16(s01, mu2), C);
-            }
-            st_half_sat(msg, sl[0], add_f16(lam, mu1));
-            st_half_sat(msg, sl[1], s0);
-            return clampc(add_f16(s0, mu1), C);
-        }
-    }
-    // The clamp is the identity unless some value exceeds C in magnitude, so it is
-    // applied only then (same values either way).  Binary16 storage with another C takes
-    // the generic loop (less code in the persistent kernel; the same sums and clamps).
-    if (sizeof(MT) == 4 && deg == 3) {
-        const float mu0 = Msg<MT>::ld(msg, sl[0]), mu1 = Msg<MT>::ld(msg, sl[1]),
-                    mu2 = Msg<MT>::ld(msg, sl[2]);
-        const float s0 = __fadd_rn(lam, mu0), s01 = __fadd_rn(s0, mu1);
-        float n0 = __fadd_rn(__fadd_rn(lam, mu1), mu2), n1 = __fadd_rn(s0, mu2), n2 = s01;
-        float L = __fadd_rn(s01, mu2);
-        if (fmaxf(fmaxf(fabsf(n0), fabsf(n1)), fmaxf(fabsf(n2), fabsf(L))) > C) {
-            n0 = clampc(n0, C);
-            n1 = clampc(n1, C);
-            n2 = clampc(n2, C);
-            L = clampc(L, C);
-        }
-        Msg<MT>::st(msg, sl[0], n0);
-        Msg<MT>::st(msg, sl[1], n1);
-        Msg<MT>::st(msg, sl[2], n2);
-        return L;
-    }
-    if (sizeof(MT) == 4 && deg == 2) {
-        const float mu0 = Msg<MT>::ld(msg, sl[0]), mu1 = Msg<MT>::ld(msg, sl[1]);
-        const float s0 = __fadd_rn(lam, mu0);
-        float n0 = __fadd_rn(lam, mu1), n1 = s0, L = __fadd_rn(s0, mu1);
-        if (fmaxf(fmaxf(fabsf(n0), fabsf(n1)), fabsf(L)) > C) {
-            n0 = clampc(n0, C);
-            n1 = clampc(n1, C);
-            L = clampc(L, C);
-        }
-        Msg<MT>::st(msg, sl[0], n0);
-        Msg<MT>::st(msg, sl[1], n1);
-        return L;
-    }
-    float mu[DV];
-#pragma unroll
-    for (int k = 0; k < DV; ++k) mu[k] = (k < deg) ? Msg<MT>::ld(msg, sl[k]) : 0.0f;
-    float L = lam;
-#pragma unroll
-    for (int k = 0; k < DV; ++k)
-        if (k < deg) L = __fadd_rn(L, mu[k]);
+    using R = Raw<MT>;
+    typename R::T mu[DV];
 #pragma unroll
     for (int k = 0; k < DV; ++k) {
-        if (k < deg) {
-            float v = lam;
-#pragma unroll
-            for (int k2 = 0; k2 < DV; ++k2)
-                if (k2 != k && k2 < deg) v = __fadd_rn(v, mu[k2]);
-            Msg<MT>::st(msg, sl[k], clampc(v, C));
-        }
+        mu[k] = 0;
+        if (k < deg) mu[k] = ld_raw<MT>(msg, sl[k]);
     }
-    return clampc(L, C);
+    float p = lam;  // lam + mu_0 + .. + mu_{k-1}
+#pragma unroll
+    for (int k = 0; k < DV; ++k) {
+        float v = p;
+#pragma unroll
+        for (int k2 = k + 1; k2 < DV; ++k2) v = R::add(v, mu[k2]);
+        if (k < deg) Msg<MT>::st(msg, sl[k], clampc(v, C));
+        p = R::add(p, mu[k]);
+    }
+    return clampc(p, C);
+}
+
+// Check of a message slot from its byte offset.
+template <typename MT, int DC>
+__device__ __forceinline__ int check_of_slot(int off) {
+    if (sizeof(MT) == 2) return 2 * (off / (4 * DC)) + ((off >> 1) & 1);
+    return off / (4 * DC);
 }
 
 // Fault pass: memory update, marginals, fault->check messages, decisions into the
 // bitmap fw, and the syndrome of the decision: every fault with F_j = 1 flips the
-// parity bits of its checks in par (zeroed by the preceding check pass).  Decisions
-// are sparse, so this costs a few atomics per shot instead of a pass over all edges.
-// Returns the thread's decided faults (bit r: fault threadIdx.x + r*NT has F_j = 1).
-template <typename MT, int NT, int VPT, int DV, bool SKIP = false>
+// parity bits of its checks in par (the preceding check pass set it to the syndrome, so
+// all words end 0 iff H F = sigma).  Decisions are sparse, so this costs a few atomics
+// per shot instead of a pass over all edges.
+// The decision of a fault is the sign bit of its marginal (never -0, see fault_update), shifted
+// into a mask; the bitmap words and the parity flips follow for the warps that decided any.
+// Returns the thread's decided faults (bit VPT-1-r: fault threadIdx.x + r*NT has F_j = 1).
+template <typename MT, int NT, int VPT, int DC, int DV>
 __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned char *msg, uint32_t *fw,
-                                           uint32_t *par, float (&Lam)[VPT],
+                                           uint32_t *par, int packed, float (&Lam)[VPT],
                                            const float (&bb)[VPT], const float (&gg)[VPT],
                                            float C) {
     static_assert(VPT <= 32, "one decision bit per fault of the thread");
-    const int lane = threadIdx.x & 31;
-    uint32_t dmask = 0u;  // bit r: this thread's fault r is decided (F_j = 1)
-#pragma unroll
-    for (int r = 0; r < VPT; ++r) {
-        if (SKIP && r * NT >= g.N) break;  // the block's remaining fault slots are empty
+    const int lane = threadIdx.x & 31, wb = threadIdx.x & ~31;
+    const uint2 *rec = Packed<MT, NT * VPT>::table(g) + threadIdx.x;
+    uint32_t dmask = 0u;
+    auto decide = [&](float L) {
+        dmask = __funnelshift_l(__float_as_uint(L), dmask, 1);  // dmask << 1 | sign(L)
+    };
+    auto fast = [&](int r) {
+        const Packed<MT, NT * VPT> s(__ldg(rec + r * NT));
+        const float lam = __fadd_rn(bb[r], __fmul_rn(gg[r], Lam[r]));
+        Lam[r] = fault_update(msg, s, lam, C);
+        decide(Lam[r]);
+    };
+    auto any = [&](int r) {
         const int j = threadIdx.x + r * NT;
-        const bool valid = j < g.N;
         float L = 0.0f;
-        if (valid) {
+        if (j < g.N) {
             const float lam = __fadd_rn(bb[r], __fmul_rn(gg[r], Lam[r]));
             int sl[DV];
             const int deg = load_slots<DV>(g, j, sl);
             L = fault_update<MT, DV>(msg, sl, deg, lam, C);
             Lam[r] = L;
         }
-        const bool dec = valid && L < 0.0f;
-        const uint32_t bal = __ballot_sync(FULL, dec);
-        const int jb = threadIdx.x - lane + r * NT;
-        if (lane == 0 && jb < g.N) fw[jb >> 5] = bal;
-        dmask |= (dec ? 1u : 0u) << r;
-    }
-    // Decided faults are few: flip their checks' parity after the loop, so that the
-    // per-fault body carries no divergent branch and no live edge state.
-    const uint32_t decided = dmask;
-    while (dmask) {
-        const int r = __ffs(dmask) - 1;
-        dmask &= dmask - 1u;
-        const int j = threadIdx.x + r * NT;
-        const int deg = (int)((uint32_t)__ldg(g.var_slot + (size_t)j * DV) >> 24);
-        const int *ck = g.var_chk + (size_t)j * DV;
-        for (int k = 0; k < deg; ++k) {
-            const int c = __ldg(ck + k);
-            atomicXor(par + (c >> 5), 1u << (c & 31));
+        decide(L);
+    };
+    each_fault<VPT>(packed, fast, any);
+    __syncwarp();
+    // bitmap words of the warp: fault slot r's 32 faults are word (wb + r NT) / 32
+    uint32_t word = 0u;
+    if (__any_sync(FULL, dmask != 0u)) {
+#pragma unroll
+        for (int r = 0; r < VPT; ++r) {
+            const uint32_t bal = __ballot_sync(FULL, (dmask >> (VPT - 1 - r)) & 1u);
+            if (lane == r) word = bal;
+        }
+        // decided faults are few: flip their checks' parity
+        for (uint32_t m = dmask; m; m &= m - 1u) {
+            const int r = VPT - __ffs(m);
+            int sl[DV];
+            const int deg = load_slots<DV>(g, threadIdx.x + r * NT, sl);
+#pragma unroll
+            for (int k = 0; k < DV; ++k)
+                if (k < deg) {
+                    const int c = check_of_slot<MT, DC>(sl[k]);
+                    atomicXor(par + (c >> 5), 1u << (c & 31));
+                }
         }
     }
-    return decided;
+    if (lane < VPT && wb + lane * NT < g.N) fw[(wb + lane * NT) >> 5] = word;
+    return dmask;
 }
 
-// H F = sigma ?  Each warp compares the parity words with the syndrome on its own
-// (no block barrier); every warp reaches the same answer.
-__device__ __forceinline__ bool warp_converged(const uint32_t *par, const uint32_t *sg, int nw) {
-    uint32_t bad = 0;
-    for (int q = threadIdx.x & 31; q < nw; q += 32) bad |= par[q] ^ sg[q];
+// H F = sigma ?  (every parity word 0)  Each warp looks on its own (no block barrier);
+// every warp reaches the same answer.
+__device__ __forceinline__ bool warp_converged(const uint32_t *par, int nw) {
+    const int lane = threadIdx.x & 31;
+    uint32_t bad = lane < nw ? par[lane] : 0u;
+    for (int q = lane + 32; q < nw; q += 32) bad |= par[q];
     return !__any_sync(FULL, bad != 0u);
 }
 
 // Adds this thread's share of the solution weight sum_j F_j w_j (2^-33 units) to the
 // block's accumulator: only the few threads with decided faults (mask dm from the
-// fault pass) issue an atomic.  Integer addition makes the total exact and
+// fault pass, bit VPT-1-r for fault r) issue an atomic.  Integer addition makes the total exact and
 // independent of the order.
-template <int NT>
-__device__ __forceinline__ void add_weight(const float *ws, uint32_t dm, long long *acc) {
+template <int NT, int VPT>
+__device__ __forceinline__ void add_weight(const FusedGraph &g, uint32_t dm, long long *acc) {
     long long w = 0;
-    for (uint32_t m = dm; m; m &= m - 1u) w += wfix(ws[threadIdx.x + (__ffs(m) - 1) * NT]);
+    for (uint32_t m = dm; m; m &= m - 1u) w += wfix(__ldg(g.w + threadIdx.x + (VPT - __ffs(m)) * NT));
     if (w != 0)
         atomicAdd(reinterpret_cast<unsigned long long *>(acc), (unsigned long long)w);
 }
@@ -483,16 +592,16 @@ __device__ __forceinline__ void keep_solution(uint64_t *dst, const uint32_t *fw,
 
 // Shared memory: messages [msg_bytes], decision bitmap fw [f_words], kept solution
 // fb [f_words], syndrome sg [2*syn_words] (bits past M cleared), two parity buffers
-// par [2][m_words], prior LLRs ws [N] (read by the weight sum and leg initialisation).
+// par [2][m_words].  (The prior LLRs are read from global memory, once a shot and for the
+// decided faults of a solution.)
 __device__ __forceinline__ void smem_layout(const FusedGraph &g, unsigned char *raw,
                                             uint32_t *&fw, uint32_t *&fb, uint32_t *&sg,
-                                            uint32_t *&par, float *&ws) {
+                                            uint32_t *&par) {
     const size_t mb = ((size_t)g.msg_bytes + 15) & ~(size_t)15;
     fw = reinterpret_cast<uint32_t *>(raw + mb);
     fb = fw + g.f_words;
     sg = fb + g.f_words;
     par = sg + 2 * g.syn_words;
-    ws = reinterpret_cast<float *>(par + 2 * g.m_words);
 }
 
 // Plain min-sum BP (paper Sec. 2.3, "Belief propagation decoding"): DMem-BP with every
@@ -503,7 +612,7 @@ __device__ __forceinline__ void smem_layout(const FusedGraph &g, unsigned char *
 template <int NT, int VPT, int DC, int DV>
 __device__ __forceinline__ void plain_bp(const FusedGraph &g, const DevParams &p, int iters,
                                          const uint64_t *sy, unsigned char *msg, uint32_t *fw,
-                                         uint32_t *sg, uint32_t *par, float *ws,
+                                         uint32_t *sg, uint32_t *par,
                                          float (&Lam)[VPT], float (&bb)[VPT], float (&gg)[VPT]);
 
 // Is the decision bitmap equal to the kept solution (its first `words` words)?  Each
@@ -523,9 +632,8 @@ __device__ __forceinline__ bool warp_same_solution(const uint32_t *fw, const uin
 // Padding slots of every check hold C for good (the check pass writes C back).
 template <typename MT, int NT, int DC>
 __device__ __forceinline__ void block_setup(const FusedGraph &g, unsigned char *msg, uint32_t *fw,
-                                            float *ws, float C) {
+                                            float C) {
     for (int q = threadIdx.x; q < 2 * g.f_words; q += NT) fw[q] = 0u;  // fw and fb
-    for (int j = threadIdx.x; j < g.N; j += NT) ws[j] = __ldg(g.w + j);
     for (int i = threadIdx.x; i < g.Mp; i += NT) {
         const int deg = g.chk_deg[i];
         const bool half = sizeof(MT) == 2;
@@ -554,17 +662,21 @@ __device__ __forceinline__ void load_syndrome(const FusedGraph &g, const uint64_
 template <int NT, int VPT, int DC, int DV>
 __device__ __forceinline__ void plain_bp(const FusedGraph &g, const DevParams &p, int iters,
                                          const uint64_t *sy, unsigned char *msg, uint32_t *fw,
-                                         uint32_t *sg, uint32_t *par, float *ws,
+                                         uint32_t *sg, uint32_t *par,
                                          float (&Lam)[VPT], float (&bb)[VPT], float (&gg)[VPT]) {
-    block_setup<float, NT, DC>(g, msg, fw, ws, p.clip);
+    block_setup<float, NT, DC>(g, msg, fw, p.clip);
     load_syndrome<NT>(g, sy, sg);
+    const int packed = packed_slots<float, NT, VPT, DV>(g);
+    RowBits rb;
+    rb.part = partial_rows<float, NT, DC>(g);
+    row_syndromes<float, NT>(g, sy, rb);
     __syncthreads();
-    leg_init<float, NT, VPT, DV>(g, p, 0, msg, ws, Lam, bb, gg);
+    leg_init<float, NT, VPT, DV>(g, p, 0, msg, packed, Lam, bb, gg);
     __syncthreads();
     for (int t = 0; t < iters; ++t) {
-        check_pass<NT, DC>(g, reinterpret_cast<float *>(msg), sg, par, p.clip);
+        check_pass<NT, DC>(g, reinterpret_cast<float *>(msg), sg, par, rb, p.clip);
         __syncthreads();
-        fault_pass<float, NT, VPT, DV>(g, msg, fw, par, Lam, bb, gg, p.clip);
+        fault_pass<float, NT, VPT, DC, DV>(g, msg, fw, par, packed, Lam, bb, gg, p.clip);
         __syncthreads();
     }
 }

@@ -33,106 +33,134 @@
 namespace qldpc {
 namespace {
 
+// Block-wide state of the shot in flight, in shared memory: the passes need nearly every
+// register of the persistent shapes, and this is read and written at leg boundaries only
+// (in registers it cost the passes 600 of 5,850 warp-instructions an iteration, in values
+// computed again; gross code, 30,000 shots at 384 threads: 1.77 -> 1.71 ms without).
+// A value that changes at a boundary has two copies, used in turn, so that the thread that
+// writes the next one never meets a reader of the last one between the same two barriers.
+struct ShotState {
+    int shot, rec;       // the shot, and its record when it is resumed
+    int slot;            // record taken for a suspension (-1: go on)
+    long long iters[2];  // iterations run before leg r: iters[r & 1]
+    long long wacc[2];   // weight of the new solution, added up by its faults' threads
+    long long best[2];   // weight of the kept solution (kNoWeight: none); copy in use: as wacc
+};
+constexpr long long kNoWeight = 0x7fffffffffffffffLL;
+
 // Relay on one shot: the leg schedule around the check and fault passes.  Per
 // iteration: check pass | barrier | fault pass | barrier | per-warp convergence
 // test.  A leg end adds the weight sum, the next leg's initialisation and one
 // barrier.  Called by every thread of the block with block-uniform arguments.
-// SKIP: the shot's code may use only part of the block's fault slots (mixed batches),
-// so the per-fault loops stop at the code's last slot.
-// wacc[2]: the block's weight accumulators, used in turn (ab selects the one the next
-// new solution adds into); the other one is zeroed after each use, at least two
-// barriers before it is added into again.  Both start at zero and ab persists across
-// the block's shots.
+// packed and rb.part: the warp's packed fault slots and the thread's rows with padding, of
+// the shot's code; the rest of rb is set here.
+// ab selects the copy of st.wacc and st.best in use; the other accumulator is zeroed after
+// each use, at least two barriers before it is added into again.  Both start at zero and
+// ab persists across the block's shots.
+// A solution is kept iff one has been found (sols > 0).
 // Tail continuation (TailCont): with tc.mode 1 a shot that reaches a leg boundary after
 // tc.cut iterations, with a next leg to run, may be suspended (its state saved in a
-// record, no outputs written); rec >= 0 resumes the shot of record rec at its boundary.
-// s_slot: a shared int that broadcasts the record taken for a suspension.
-template <typename MT, int NT, int VPT, int DC, int DV, bool SKIP = false, bool RESUME = false>
-__device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams &p, int shot,
-                                            const uint64_t *sy, uint64_t *cor, DecodeOut out,
+// record, no outputs written); RESUME takes the shot of record st.rec up at its boundary.
+template <typename MT, int NT, int VPT, int DC, int DV, bool RESUME = false>
+__device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams &p,
+                                            const uint64_t *__restrict__ syn, int syn_stride,
+                                            int cor_stride, const DecodeOut &out,
                                             unsigned char *msg, uint32_t *fw, uint32_t *fb,
-                                            uint32_t *sg, uint32_t *par, float *ws,
-                                            long long *wacc,
+                                            uint32_t *sg, uint32_t *par, ShotState &st, int packed, RowBits &rb,
                                             float (&Lam)[VPT], float (&bb)[VPT],
-                                            float (&gg)[VPT], int &ab, const TailCont &tc,
-                                            int rec, int *s_slot) {
+                                            float (&gg)[VPT], int &ab, const TailCont &tc) {
     const int tid = threadIdx.x;
     const float C = p.clip;
-    load_syndrome<NT>(g, sy, sg);
-    int leg = 0, sols = 0, t = 0, pb = 0;
-    long long iters = 0, Wbest = 0;
-    bool have = false;
+    int leg = 0, sols = 0;
+    {
+        const uint64_t *sy = syn + (size_t)st.shot * syn_stride;
+        load_syndrome<NT>(g, sy, sg);
+        row_syndromes<MT, NT>(g, sy, rb);
+    }
     if (RESUME) {  // resume at the boundary where the first launch stopped the shot
-        const TailRecord r = tc.rec[rec];
+        const TailRecord r = tc.rec[st.rec];
         leg = r.leg;
         sols = r.sols;
-        have = r.have != 0;
-        iters = r.iters;
-        Wbest = r.Wbest;
-        const float *lr = tc.lam + (size_t)rec * g.N;
+        if (tid == 0) {
+            st.iters[leg & 1] = r.iters;
+            st.best[ab] = r.have ? r.Wbest : kNoWeight;
+        }
+        const float *lr = tc.lam + (size_t)st.rec * g.N;
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
             const int j = threadIdx.x + q * NT;
             if (j < g.N) Lam[q] = lr[j];
         }
-        if (have)  // the kept solution, for the same-solution test
+        if (sols > 0) {  // the kept solution, for the same-solution test
+            const uint64_t *cor = out.corr + (size_t)st.shot * cor_stride;
             for (int q = tid; q < g.cor_words; q += NT) {
                 const uint64_t v = cor[q];
                 fb[2 * q] = (uint32_t)v;
                 fb[2 * q + 1] = (uint32_t)(v >> 32);
             }
-    }
-    leg_init<MT, NT, VPT, DV, SKIP>(g, p, leg, msg, ws, Lam, bb, gg);
-    __syncthreads();
-    for (;;) {
-        uint32_t *pc = par + pb * g.m_words;
-        check_pass<NT, DC>(g, reinterpret_cast<MT *>(msg), sg, pc, C);
-        __syncthreads();
-        const uint32_t dm = fault_pass<MT, NT, VPT, DV, SKIP>(g, msg, fw, pc, Lam, bb, gg, C);
-        __syncthreads();
-        ++iters;
-        ++t;
-        pb ^= 1;
-        const bool conv = warp_converged(pc, sg, g.m_words);
-        const bool spent = p.max_iters > 0 && iters >= p.max_iters;
-        const bool leg_end = conv || spent || t == (leg == 0 ? p.T1 : p.T2);
-        if (!leg_end) continue;
-        // a solution equal to the kept one has its weight and cannot replace it
-        const bool fresh = conv && !(have && warp_same_solution(fw, fb, 2 * g.cor_words));
-        if (conv) ++sols;
-        if (fresh) add_weight<NT>(ws, dm, wacc + ab);
-        const bool done = sols >= p.S || leg == p.R || spent;
-        if (!done) {
-            ++leg;
-            t = 0;
-            leg_init<MT, NT, VPT, DV, SKIP>(g, p, leg, msg, ws, Lam, bb, gg);
         }
+    } else if (tid == 0) {
+        st.iters[0] = 0;
+        st.best[ab] = kNoWeight;
+    }
+    // each pass of this loop starts at a leg boundary: the next leg's initial messages, one
+    // barrier, the kept solution's update, then the leg's iterations
+    uint32_t *pc = par;  // this iteration's parity words: the two buffers take turns
+    bool fresh = false, done = false;
+    for (;;) {
+        if (!done) leg_init<MT, NT, VPT, DV>(g, p, leg, msg, packed, Lam, bb, gg);
         // a long shot with a next leg to run is suspended if a record is free (the next
         // leg's initialisation is redone on resumption from the same state); thread 0
-        // decides and takes the record, *s_slot tells the block (-1: go on)
+        // decides and takes the record, st.slot tells the block (-1: go on)
         if (!RESUME && tid == 0) {
             int k = -1;
-            if (!done && tc.mode == 1 && iters >= tc.cut) {
+            if (!done && tc.mode == 1 && st.iters[leg & 1] >= tc.cut) {
                 const unsigned int c = atomicAdd(tc.count, 1u);
                 if (c < (unsigned int)tc.cap) k = (int)c;
             }
-            *s_slot = k;
+            st.slot = k;
         }
-        __syncthreads();  // the weight and the next leg's initial messages are visible
+        __syncthreads();  // the weight and the leg's initial messages are visible
         if (fresh) {
-            const long long W = wacc[ab];
-            if (!have || W < Wbest) {
-                keep_solution<NT>(cor, fw, fb, g.cor_words);
-                have = true;
-                Wbest = W;
+            const long long W = st.wacc[ab], best = st.best[ab];
+            if (W < best)
+                keep_solution<NT>(out.corr + (size_t)st.shot * cor_stride, fw, fb, g.cor_words);
+            if (tid == 0) {
+                st.wacc[ab ^ 1] = 0;
+                st.best[ab ^ 1] = W < best ? W : best;
             }
-            if (tid == 0) wacc[ab ^ 1] = 0;
             ab ^= 1;
         }
-        if (!RESUME && *s_slot >= 0) break;
+        if (!RESUME && st.slot >= 0) break;
         if (done) break;
+        // iterations this leg may run: its limit and what the budget leaves
+        int limit = leg == 0 ? p.T1 : p.T2;
+        if (p.max_iters > 0) {
+            const long long left = p.max_iters - st.iters[leg & 1];
+            limit = left < limit ? (left < 1 ? 1 : (int)left) : limit;
+        }
+        uint32_t dm;
+        bool conv;
+        int t = 0;
+        do {
+            check_pass<NT, DC>(g, reinterpret_cast<MT *>(msg), sg, pc, rb, C);
+            __syncthreads();
+            dm = fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, pc, packed, Lam, bb, gg, C);
+            __syncthreads();
+            ++t;
+            conv = warp_converged(pc, g.m_words);
+            pc = pc == par ? par + g.m_words : par;
+        } while (!conv && t != limit);
+        // a solution equal to the kept one has its weight and cannot replace it
+        fresh = conv && !(sols > 0 && warp_same_solution(fw, fb, 2 * g.cor_words));
+        if (conv) ++sols;
+        if (fresh) add_weight<NT, VPT>(g, dm, st.wacc + ab);
+        const long long iters = st.iters[leg & 1] + t;
+        done = sols >= p.S || leg == p.R || (p.max_iters > 0 && iters >= p.max_iters);
+        if (tid == 0) st.iters[(leg + 1) & 1] = iters;
+        ++leg;
     }
-    const int slot = RESUME ? -1 : *s_slot;  // this shot's last leg end set it
+    const int slot = RESUME ? -1 : st.slot;  // this shot's last leg boundary set it
     if (slot >= 0) {  // suspended: the state at this boundary; the next leg runs on resumption
         float *lr = tc.lam + (size_t)slot * g.N;
 #pragma unroll
@@ -140,14 +168,16 @@ __device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams
             const int j = threadIdx.x + q * NT;
             if (j < g.N) lr[j] = Lam[q];
         }
-        if (tid == 0) tc.rec[slot] = TailRecord{shot, leg, sols, have ? 1 : 0, iters, Wbest};
+        if (tid == 0)
+            tc.rec[slot] = TailRecord{st.shot, leg, sols, sols > 0 ? 1 : 0, st.iters[leg & 1],
+                                      st.best[ab]};
         return;
     }
-    if (!have) store_bits<NT>(cor, fw, g.cor_words);
+    if (sols == 0) store_bits<NT>(out.corr + (size_t)st.shot * cor_stride, fw, g.cor_words);
     if (tid == 0) {
-        if (out.legs) out.legs[shot] = leg + 1;
-        if (out.conv) out.conv[shot] = have ? 1 : 0;
-        if (out.iters) out.iters[shot] = (int32_t)iters;
+        if (out.legs) out.legs[st.shot] = leg;
+        if (out.conv) out.conv[st.shot] = sols > 0 ? 1 : 0;
+        if (out.iters) out.iters[st.shot] = (int32_t)st.iters[leg & 1];
     }
 }
 
@@ -163,40 +193,38 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode(FusedGraph g, DevParams
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *msg = smem_raw;
     uint32_t *fw, *fb, *sg, *par;
-    float *ws;
-    smem_layout(g, smem_raw, fw, fb, sg, par, ws);
-    __shared__ int s_shot, s_rec, s_slot;
-    __shared__ long long s_wacc[2];
-    block_setup<MT, NT, DC>(g, msg, fw, ws, p.clip);
+    smem_layout(g, smem_raw, fw, fb, sg, par);
+    __shared__ ShotState st;
+    block_setup<MT, NT, DC>(g, msg, fw, p.clip);
+
+    const int packed = packed_slots<MT, NT, VPT, DV>(g);
+    RowBits rb;
+    rb.part = partial_rows<MT, NT, DC>(g);
 
     float Lam[VPT], bb[VPT], gg[VPT];
 #pragma unroll
     for (int r = 0; r < VPT; ++r) Lam[r] = bb[r] = gg[r] = 0.0f;
     int ab = 0;
-    if (threadIdx.x < 2) s_wacc[threadIdx.x] = 0;
+    if (threadIdx.x < 2) st.wacc[threadIdx.x] = 0;
 
     const int limit = RESUME ? (int)min(*tc.count, (unsigned int)tc.cap)
                              : (map.order ? min(*map.count, B) : B);
     for (;;) {
-        __syncthreads();  // the previous shot is done with shared memory and s_shot
+        __syncthreads();  // the previous shot is done with shared memory and its state
         if (threadIdx.x == 0) {
             const int k = (int)atomicAdd(counter, 1u);
             if (RESUME) {
-                s_rec = k < limit ? k : -1;
-                s_shot = k < limit ? tc.rec[k].shot : -1;
+                st.rec = k;
+                st.shot = k < limit ? tc.rec[k].shot : -1;
             } else {
-                s_rec = -1;
-                s_shot = k < limit ? (map.order ? map.order[k] : k) : -1;
+                st.shot = k < limit ? (map.order ? map.order[k] : k) : -1;
             }
         }
         __syncthreads();
-        const int shot = s_shot;
-        if (shot < 0) break;
-        decode_shot<MT, NT, VPT, DC, DV, false, RESUME>(g, p, shot,
-                                         syn + (size_t)shot * map.syn_stride,
-                                         out.corr + (size_t)shot * map.cor_stride, out, msg, fw,
-                                         fb, sg, par, ws, s_wacc, Lam, bb, gg, ab, tc, s_rec,
-                                         &s_slot);
+        if (st.shot < 0) break;
+        decode_shot<MT, NT, VPT, DC, DV, RESUME>(g, p, syn, map.syn_stride, map.cor_stride, out,
+                                                 msg, fw, fb, sg, par, st, packed, rb, Lam,
+                                                 bb, gg, ab, tc);
     }
 }
 
@@ -213,21 +241,24 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode_multi(MultiTable tab,
     unsigned char *msg = smem_raw;
     __shared__ FusedGraph s_g;
     __shared__ DevParams s_p;
-    __shared__ int s_shot, s_code, s_slot;
-    __shared__ long long s_wacc[2];
+    __shared__ ShotState st;
+    __shared__ int s_code;
     int cur = -1;
+    int packed = 0;
+    RowBits rb;
+    rb.part = 0u;
 
     float Lam[VPT], bb[VPT], gg[VPT];
 #pragma unroll
     for (int r = 0; r < VPT; ++r) Lam[r] = bb[r] = gg[r] = 0.0f;
     int ab = 0;
-    if (threadIdx.x < 2) s_wacc[threadIdx.x] = 0;
+    if (threadIdx.x < 2) st.wacc[threadIdx.x] = 0;
 
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) {
             const int shot = (int)atomicAdd(counter, 1u);
-            s_shot = shot;
+            st.shot = shot;
             int c = shot < B ? code_of_shot[shot] : 0;
             if (c < 0 || c >= tab.n) c = -1;  // invalid code id: the shot is skipped
             s_code = c;
@@ -237,7 +268,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode_multi(MultiTable tab,
             }
         }
         __syncthreads();
-        const int shot = s_shot, code = s_code;
+        const int shot = st.shot, code = s_code;
         if (shot >= B) break;
         if (code < 0) {  // not a code of the table: marked by iters = -1
             if (threadIdx.x == 0) {
@@ -248,17 +279,17 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode_multi(MultiTable tab,
             continue;
         }
         uint32_t *fw, *fb, *sg, *par;
-        float *ws;
-        smem_layout(s_g, smem_raw, fw, fb, sg, par, ws);
+            smem_layout(s_g, smem_raw, fw, fb, sg, par);
         if (code != cur) {
-            block_setup<MT, NT, DC>(s_g, msg, fw, ws, s_p.clip);
+            block_setup<MT, NT, DC>(s_g, msg, fw, s_p.clip);
+            packed = packed_slots<MT, NT, VPT, DV>(s_g);
+            rb.part = partial_rows<MT, NT, DC>(s_g);
             cur = code;
             __syncthreads();
         }
-        decode_shot<MT, NT, VPT, DC, DV, true>(s_g, s_p, shot, syn + (size_t)shot * syn_stride,
-                                         out.corr + (size_t)shot * cor_stride, out, msg, fw, fb,
-                                         sg, par, ws, s_wacc, Lam, bb, gg, ab, TailCont{},
-                                         -1, &s_slot);
+        decode_shot<MT, NT, VPT, DC, DV>(s_g, s_p, syn, syn_stride, cor_stride, out, msg, fw, fb,
+                                         sg, par, st, packed, rb, Lam, bb, gg, ab,
+                                         TailCont{});
     }
 }
 
@@ -270,22 +301,25 @@ __global__ void __launch_bounds__(NT) fused_trace(FusedGraph g, DevParams p,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *msg = smem_raw;
     uint32_t *fw, *fb, *sg, *par;
-    float *ws;
-    smem_layout(g, smem_raw, fw, fb, sg, par, ws);
+    smem_layout(g, smem_raw, fw, fb, sg, par);
     const int shot = blockIdx.x;
     const float C = p.clip;
-    block_setup<MT, NT, DC>(g, msg, fw, ws, C);
+    block_setup<MT, NT, DC>(g, msg, fw, C);
     load_syndrome<NT>(g, syn + (size_t)shot * g.syn_words, sg);
     float Lam[VPT], bb[VPT], gg[VPT];
 #pragma unroll
     for (int r = 0; r < VPT; ++r) Lam[r] = bb[r] = gg[r] = 0.0f;
+    const int packed = packed_slots<MT, NT, VPT, DV>(g);
+    RowBits rb;
+    rb.part = partial_rows<MT, NT, DC>(g);
+    row_syndromes<MT, NT>(g, syn + (size_t)shot * g.syn_words, rb);
     __syncthreads();
-    leg_init<MT, NT, VPT, DV>(g, p, 0, msg, ws, Lam, bb, gg);
+    leg_init<MT, NT, VPT, DV>(g, p, 0, msg, packed, Lam, bb, gg);
     __syncthreads();
     const int nslots = g.msg_bytes / (int)sizeof(MT);
     for (int t = 0; t < T; ++t) {
         const size_t o = (size_t)t * B + shot;
-        check_pass<NT, DC>(g, reinterpret_cast<MT *>(msg), sg, par, C);
+        check_pass<NT, DC>(g, reinterpret_cast<MT *>(msg), sg, par, rb, C);
         __syncthreads();
         if (mu)
             for (int s = threadIdx.x; s < nslots; s += NT) {
@@ -293,7 +327,7 @@ __global__ void __launch_bounds__(NT) fused_trace(FusedGraph g, DevParams p,
                 if (e >= 0) mu[o * E + e] = Msg<MT>::ld(msg, s * (int)sizeof(MT));
             }
         __syncthreads();
-        fault_pass<MT, NT, VPT, DV>(g, msg, fw, par, Lam, bb, gg, C);
+        fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, par, packed, Lam, bb, gg, C);
         __syncthreads();
         if (marg) {
 #pragma unroll
@@ -305,7 +339,9 @@ __global__ void __launch_bounds__(NT) fused_trace(FusedGraph g, DevParams p,
         if (nu)
             for (int s = threadIdx.x; s < nslots; s += NT) {
                 const int e = g.slot_edge[s];
-                if (e >= 0) nu[o * E + e] = Msg<MT>::ld(msg, s * (int)sizeof(MT));
+                if (e < 0) continue;
+                const float x = Msg<MT>::ld(msg, s * (int)sizeof(MT));  // stored unclamped
+                nu[o * E + e] = fabsf(x) > C ? copysignf(C, x) : x;
             }
         __syncthreads();
     }

@@ -1,0 +1,77 @@
+"""Paths of the decode kernels' check and fault passes, against the oracle mirror bit for bit:
+packed slot records and the general fault path in one warp, rows with no, one or several
+padding slots, saturated messages, and the recorded messages of the first leg."""
+import numpy as np
+import pytest
+
+from oracle.relay import RelayParams, dmem_trace, relay_decode
+from workloads import DecodingProblem, pack_bits
+
+from _cases import assert_same_decisions, gamma_for, gpu_decode, syndrome
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+from paper_2511_21660_gb300 import (QLDPC_MSG_FP16, QLDPC_MSG_FP32, RelayConfig,  # noqa: E402
+                                    RelayDecoder)
+
+PREC = {QLDPC_MSG_FP32: "f32", QLDPC_MSG_FP16: "f16s"}
+
+
+def _graph(rng, M, N, degrees, dc):
+    """Random H with fault degrees drawn from `degrees` and check degrees at most dc (a fault
+    that finds no room keeps fewer checks)."""
+    H = np.zeros((M, N), dtype=np.uint8)
+    for j in range(N):
+        room = np.nonzero(H.sum(1) < dc)[0]
+        d = min(int(rng.choice(degrees)), room.size)
+        H[rng.choice(room, d, replace=False), j] = 1
+    return H
+
+
+# (checks, faults, fault degrees, check degree): whole warps of degree 2 and 3; a ragged last
+# warp; degrees 0..4 mixed in every warp; sparse rows (many padding slots, empty rows);
+# the 16- and 32-slot families with their 8 fault slots
+GRAPHS = [(160, 384, (2, 3), 8), (161, 385, (3,), 8), (130, 301, (0, 1, 2, 3, 4), 8),
+          (300, 320, (1, 2), 8), (120, 416, (2, 3), 16), (60, 351, (1, 2, 3, 5, 8), 32)]
+
+
+@pytest.mark.parametrize("M,N,degrees,dc", GRAPHS)
+@pytest.mark.parametrize("prec", [QLDPC_MSG_FP32, QLDPC_MSG_FP16])
+@pytest.mark.parametrize("clip", [0.0, 12.0])
+def test_random_graphs_match_the_mirror(M, N, degrees, dc, prec, clip):
+    rng = np.random.default_rng(M * 1000 + N)
+    H = _graph(rng, M, N, degrees, dc)
+    p = rng.uniform(0.005, 0.08, N)
+    P = DecodingProblem("random", H, np.zeros((1, N), np.uint8), p, {"code": "bb72"})
+    sig = syndrome(P, (rng.random((150, N)) < p).astype(np.uint8))
+    sig[:20] = rng.random((20, M)) < 0.5                   # mostly unsolvable: many legs
+    gam = gamma_for(P, R=8, seed=N)
+    cfg = dict(legs_after_first=8, iters_first=20, iters_later=15, stop_after_solutions=3)
+    got = gpu_decode(P, gam, sig, RelayConfig(msg_precision=prec, llr_clip=clip, **cfg))
+    prm = RelayParams(**cfg)
+    if clip:
+        prm.clip = clip
+    ref = relay_decode(P.row_ptr, P.col_idx, P.p, gam, sig, prm, precision=PREC[prec])
+    assert_same_decisions(got, ref, f"{M}x{N}/{PREC[prec]}/{clip}")
+
+
+@pytest.mark.parametrize("prec", [QLDPC_MSG_FP32, QLDPC_MSG_FP16])
+def test_recorded_messages_saturate_like_the_oracle(prec):
+    """The passes hold fault-to-check messages unclamped; the trace records them clamped."""
+    rng = np.random.default_rng(8)
+    H = _graph(rng, 161, 385, (2, 3), 8)
+    P = DecodingProblem("random", H, np.zeros((1, 385), np.uint8), rng.uniform(0.005, 0.08, 385),
+                        {"code": "bb72"})
+    sig = (rng.random((16, 161)) < 0.3).astype(np.uint8)
+    gam = gamma_for(P, R=0)
+    dec = RelayDecoder(P.row_ptr, P.col_idx, P.p, gam,
+                       RelayConfig(legs_after_first=0, msg_precision=prec, llr_clip=12.0))
+    marg, nu, mu = dec.trace_first_leg(torch.from_numpy(pack_bits(sig).view(np.int64)).cuda(), 12)
+    torch.cuda.synchronize()
+    dec.close()
+    L, n, m = dmem_trace(P.row_ptr, P.col_idx, P.p, gam[0], sig, 12, precision=PREC[prec],
+                         clip=12.0)
+    assert np.abs(n).max() == 12.0
+    for a, b in ((marg, L), (nu, n), (mu, m)):
+        assert (a.cpu().numpy().transpose(1, 0, 2) == b).all()
