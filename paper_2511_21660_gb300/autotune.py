@@ -19,7 +19,7 @@ import numpy as np
 
 from .qldpc import QldpcError, RelayConfig, RelayDecoder
 
-CANDIDATES = (256, 384, 512, 640, 768, 1024)
+CANDIDATES = (32, 64, 128, 256, 384, 512, 640, 768, 1024)
 TAIL_OPTIONS = (0, -1)   # the library default (continuation after T_1 + 8 T_r), off
 CACHE = os.path.join(os.path.expanduser("~"), ".cache", "qldpc", "tuning.json")
 

@@ -63,6 +63,12 @@ struct qldpc_decoder {
     int msg_fp16 = 0;
     const qldpc::FusedKernel *fk = nullptr;        // decode kernel
     const qldpc::FusedKernel *fk_trace = nullptr;  // trace kernel
+    // shape for small batches (nullptr: fk serves them), its grid, and the largest such batch
+    const qldpc::FusedKernel *fk_small = nullptr;
+    int small_grid = 0;
+    int64_t small_max = 0;
+    const qldpc::FusedKernel *table = nullptr;     // compiled shapes of the decoder's family
+    int ntable = 0;
     size_t trace_smem = 0;
     int block_threads = 0, blocks_per_sm = 0, num_sms = 0, grid = 0;
     size_t smem = 0;

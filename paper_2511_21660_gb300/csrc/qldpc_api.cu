@@ -199,6 +199,32 @@ bool holds(const FusedKernel &k, int M, int N) {
     return (long long)k.threads * k.vpt >= N && 32LL * k.threads >= rows;
 }
 
+// Small batches: with fewer shots than about twice the blocks that a wider shape keeps
+// resident, a shot's latency counts and the narrow shape's full residency does not.
+// Measured (us a launch, narrow / wide): gross code 100 shots 39.5 / 34.3, 608 101 / 87, 2400
+// 145 / 165; 720 faults 608 39 / 31, 2400 56 / 67; 8064 faults 304 112 / 101, 1200 283 / 288;
+// 72 faults 2400 141 / 107.
+int setup_small(qldpc_decoder *d) {
+    for (int q = 0; q < d->ntable && !d->fk_small; ++q)
+        if (d->table[q].latency && holds(d->table[q], d->M, d->N)) d->fk_small = &d->table[q];
+    if (!d->fk_small || d->fk_small->threads <= d->fk->threads) {
+        d->fk_small = nullptr;
+        return QLDPC_OK;
+    }
+    int bps = 0;
+    QL_CUDA(cudaFuncSetAttribute(d->fk_small->decode_fn,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem));
+    QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, d->fk_small->decode_fn,
+                                                          d->fk_small->threads, d->smem));
+    if (bps < 1) {
+        d->fk_small = nullptr;
+        return QLDPC_OK;
+    }
+    d->small_grid = d->num_sms * bps;
+    d->small_max = 2LL * d->small_grid;
+    return QLDPC_OK;
+}
+
 // Tail continuation: the resuming launch runs the compiled 1024-thread shape with the
 // fewest faults per thread that holds N (one block per SM; none holds it: no
 // continuation); 4 records per SM.  tail_cut < 0 turns it off, 0 picks T_1 + 8 T_r.
@@ -244,6 +270,8 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
         if (holds(tab[q], M, N) &&
             (block_threads == 0 || tab[q].threads == block_threads))
             d->fk = &tab[q];
+    d->table = tab;
+    d->ntable = ntab;
     if (!d->fk)
         return fail(QLDPC_ERR_UNSUPPORTED, "no compiled kernel for N = %d with %d threads", N,
                     block_threads);
@@ -337,6 +365,10 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     }
     d->block_threads = d->fk->threads;
     d->grid = d->num_sms * d->blocks_per_sm;
+    if (block_threads == 0) {
+        rc = setup_small(d);
+        if (rc) return rc;
+    }
 
     // one device arena for every graph array
     const size_t R1 = (size_t)d->prm.R + 1;
@@ -433,9 +465,11 @@ int launch_persistent(const qldpc_decoder *d, const uint64_t *syn, int64_t B, De
     const bool tail = d->fk_tail != nullptr;
     QL_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned int), st));
     if (tail) QL_CUDA(cudaMemsetAsync(d->counter + 1, 0, 2 * sizeof(unsigned int), st));
-    const int grid = (int)std::min<int64_t>(d->grid, B);
-    QL_CUDA(d->fk->launch_decode(dim3(grid), d->smem, st, d->fg, d->prm, syn, (int)B, out,
-                                 counter, map, d->tail));
+    const bool small = d->fk_small && B <= d->small_max;
+    const FusedKernel *fk = small ? d->fk_small : d->fk;
+    const int grid = (int)std::min<int64_t>(small ? d->small_grid : d->grid, B);
+    QL_CUDA(fk->launch_decode(dim3(grid), d->smem, st, d->fg, d->prm, syn, (int)B, out, counter,
+                              map, d->tail));
     if (tail)
         QL_CUDA(d->fk_tail->launch_resume(dim3(std::min(d->tail_grid, d->tail.cap)), d->smem, st,
                                           d->fg, d->prm, syn, (int)B, out, d->counter + 2, map,
@@ -703,9 +737,17 @@ int qldpc_decode_batch_multi(qldpc_decoder *const *decoders, int32_t n_codes,
     for (int q = 0; q < 6; ++q)
         if (ptrs[q] && !is_device_ptr(ptrs[q]))
             return fail(QLDPC_ERR_INVALID_ARG, "argument %d is not device memory", q);
-    // the kernel instance of the code with the most faults serves every code
+    // one shape serves every code: the largest code's wide one (small codes leave most of a
+    // narrow block's fault slots empty), or the first that holds every code
     const qldpc_decoder *db = decoders[big];
-    const FusedKernel *fk = db->fk;
+    const FusedKernel *fk = db->fk_small ? db->fk_small : db->fk;
+    auto holds_all = [&](const FusedKernel &k) {
+        for (int c = 0; c < n_codes; ++c)
+            if (!holds(k, decoders[c]->M, decoders[c]->N)) return false;
+        return true;
+    };
+    for (int q = 0; q < db->ntable && !holds_all(*fk); ++q) fk = &db->table[q];
+    if (!holds_all(*fk)) return fail(QLDPC_ERR_UNSUPPORTED, "no compiled kernel holds every code");
     MultiTable tab{};
     tab.n = n_codes;
     size_t smem = 0;

@@ -379,9 +379,12 @@ using MsgT = __half;
 using MsgT = float;
 #endif
 
-template <int NT, int VPT, int MINB, bool TRACE>
+constexpr bool kLatency = QL_DC == 8;
+
+template <int NT, int VPT, int MINB, bool TRACE, bool LATENCY = false>
 FusedKernel entry() {
     FusedKernel k;
+    k.latency = LATENCY;
     k.msg_fp16 = QL_MSG_F16;
     k.threads = NT;
     k.min_blocks = MINB;
@@ -420,19 +423,54 @@ FusedKernel entry() {
 #endif
 
 void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
-    // (threads, faults per thread, min resident blocks): the first entry whose
-    // threads * vpt >= N is used unless the caller asks for a block size; the last
+    // (threads, faults per thread, min resident blocks): the first entry that holds the graph
+    // (threads * vpt >= N) is used unless the caller asks for a block size; the last
     // entry also serves the trace kernel; the 1024-thread entries serve the resuming
-    // launch of the tail continuation.
+    // launch of the tail continuation; the entries marked kLatency serve small batches.
+    //
+    // Rows of up to 8 slots: the blocks are narrow, with as many faults per thread as the
+    // registers hold at full residency, since the cost of an iteration that does not depend
+    // on the faults (barriers, the convergence test, the check pass's uneven rows) is per
+    // warp.  Each entry's reach is chosen so that the graphs it is used for fill all fault
+    // slots but the last (each_fault).  Measured, old shape -> this one: 72 faults 256 x 4 ->
+    // 32 x 3 2.26 -> 0.59 ms (60,000 shots), 720 faults 256 x 4 -> 64 x 12 1.13 -> 0.75 ms,
+    // gross code 512 x 6 -> 256 x 11 1.88 -> 1.59 ms (30,000), 8064 faults 1024 x 8 -> 256 x
+    // 32 1.72 -> 1.49 ms (8,000).
     static const FusedKernel table[] = {
-        entry<256, 4, 4, false>(),
-        entry<512, 6, 2, false>(),
+#if QL_DC == 8
+        entry<32, 3, 32, false>(),
+        entry<64, 4, 16, false, kLatency>(),
+        entry<64, 8, 16, false>(),
+        entry<64, 12, 16, false>(),
+        entry<64, 13, 12, false>(),
+        entry<128, 8, 8, false>(),
+#endif
+        entry<256, 4, 4, false, kLatency>(),
+#if QL_DC == 8
+        entry<128, 10, 6, false>(),
+        entry<128, 12, 6, false>(),
+        entry<128, 15, 5, false>(),
+        entry<128, 18, 5, false>(),
+        entry<256, 10, 4, false>(),
+        entry<256, 11, 4, false>(),
+        entry<256, 12, 4, false>(),
+#endif
+        entry<512, 6, 2, false, kLatency>(),
         entry<256, 12, 4, false>(),
         entry<384, 8, 3, false>(),
         entry<640, 5, 2, false>(),
         entry<768, 4, 2, false>(),
         entry<1024, 3, 1, false>(),
-        entry<1024, 8, 1, false>(),
+#if QL_DC == 8
+        entry<256, 14, 3, false>(),
+        entry<256, 16, 3, false>(),
+        entry<256, 18, 3, false>(),
+        entry<256, 22, 2, false>(),
+        entry<256, 25, 2, false>(),
+        entry<384, 18, 2, false>(),
+        entry<256, 32, 2, false>(),
+#endif
+        entry<1024, 8, 1, false, kLatency>(),
         entry<512, 16, 1, false>(),
         entry<512, 32, 1, true>(),
     };

@@ -5,9 +5,9 @@ import numpy as np
 import pytest
 
 from oracle.relay import RelayParams, dmem_trace, relay_decode
-from workloads import DecodingProblem, pack_bits
+from workloads import BB72, BB144, BB288, DecodingProblem, pack_bits, phenomenological_dem
 
-from _cases import assert_same_decisions, gamma_for, gpu_decode, syndrome
+from _cases import assert_same_decisions, gamma_for, gpu_decode, shots, syndrome
 
 pytestmark = pytest.mark.gpu
 
@@ -75,3 +75,51 @@ def test_recorded_messages_saturate_like_the_oracle(prec):
     assert np.abs(n).max() == 12.0
     for a, b in ((marg, L), (nu, n), (mu, m)):
         assert (a.cpu().numpy().transpose(1, 0, 2) == b).all()
+
+
+# (code, rounds, shape the library takes): each compiled shape at a graph it is used for
+SHAPES = [(BB72, 1, 64), (BB72, 4, 64), (BB72, 6, 64), (BB72, 7, 64), (BB72, 8, 128),
+          (BB72, 10, 128), (BB72, 12, 128), (BB144, 8, 128), (BB144, 10, 128), (BB144, 11, 256),
+          (BB144, 12, 256), (BB144, 13, 256), (BB144, 15, 256), (BB144, 18, 256),
+          (BB144, 20, 256), (BB288, 12, 256), (BB288, 14, 256), (BB288, 15, 384),
+          (BB288, 18, 256)]
+
+
+@pytest.mark.parametrize("code,rounds,threads", SHAPES)
+@pytest.mark.parametrize("prec", [QLDPC_MSG_FP32, QLDPC_MSG_FP16])
+def test_library_shapes_match_the_mirror(code, rounds, threads, prec):
+    """A batch above the small-batch shape's reach runs the narrow shape; its first shots are
+    the oracle's, and the whole batch is the one a 1024-thread block decodes; a small batch
+    (the wide shape) gives the same rows."""
+    P = phenomenological_dem(code, rounds, 0.006)
+    P.meta["code"] = "bb288" if code is BB288 else "bb144"
+    n, few = 5000 if code is BB72 else 1300, 40
+    sig = shots(P, n, rounds)[1]
+    gam = gamma_for(P, R=40, seed=rounds)
+    cfg = dict(legs_after_first=40, stop_after_solutions=3)
+    got = gpu_decode(P, gam, sig, RelayConfig(msg_precision=prec, **cfg))
+    assert got[4].block_threads == threads
+    ref = relay_decode(P.row_ptr, P.col_idx, P.p, gam, sig[:few], RelayParams(**cfg),
+                       precision=PREC[prec])
+    assert_same_decisions(tuple(x[:few] for x in got[:4]), ref, "library's shape")
+    wide = gpu_decode(P, gam, sig, RelayConfig(msg_precision=prec, block_threads=1024, **cfg))
+    small = gpu_decode(P, gam, sig[:few], RelayConfig(msg_precision=prec, **cfg))
+    for a, b, c in zip(got[:4], wide[:4], small[:4]):
+        assert np.array_equal(a, b) and np.array_equal(a[:few], c)
+
+
+def test_few_faults_with_many_checks_take_a_wide_enough_block():
+    """90 faults and 1,200 checks: a 32-thread block would have more rows than a thread keeps
+    syndrome bits for."""
+    rng = np.random.default_rng(5)
+    H = _graph(rng, 1200, 90, (2, 3, 4), 8)
+    P = DecodingProblem("tall", H, np.zeros((1, 90), np.uint8), np.full(90, 0.05),
+                        {"code": "bb72"})
+    sig = syndrome(P, (rng.random((200, 90)) < 0.05).astype(np.uint8))
+    gam = gamma_for(P, R=4, seed=2)
+    cfg = dict(legs_after_first=4, stop_after_solutions=2)
+    for prec in (QLDPC_MSG_FP32, QLDPC_MSG_FP16):
+        got = gpu_decode(P, gam, sig, RelayConfig(msg_precision=prec, **cfg))
+        ref = relay_decode(P.row_ptr, P.col_idx, P.p, gam, sig, RelayParams(**cfg),
+                           precision=PREC[prec])
+        assert_same_decisions(got, ref, f"tall/{PREC[prec]}")
