@@ -25,16 +25,12 @@ __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C,
                                                    const uint64_t *sy, unsigned char *msg,
                                                    uint32_t *sg, uint32_t *par,
                                                    float (&Lam)[VPT]) {
-    // padding slots hold C for good (the check pass writes C back)
-    for (int i = threadIdx.x; i < g.Mp; i += NT) {
-        const int deg = g.chk_deg[i], f = swz<DC>(i);
-        for (int k = deg; k < DC; ++k) Msg<float>::st(msg, (i * DC + (k ^ f)) * 4, C);
-    }
     load_syndrome<NT>(g, sy, sg);
-    const int packed = packed_slots<float, NT, VPT, DV>(g);
-    RowBits rb;
-    rb.part = partial_rows<float, NT, DC>(g);
     const uint2 *rec = Packed<float, NT * VPT>::table(g) + threadIdx.x;
+    FaultSlots<float, NT, VPT> fs;
+    fs.init(g);
+    RowBits rb;
+    rb.part = setup_rows<float, NT, DC>(g, msg, C);
     // nu(0) = lambda(0) = w on every edge, Lambda(0) = w
     float wr[VPT];
 #pragma unroll
@@ -58,8 +54,7 @@ __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C,
         check_pass<NT, DC>(g, reinterpret_cast<float *>(msg), sg, par, rb, C);
         __syncthreads();
         auto fast = [&](int r) {
-            const Packed<float, NT * VPT> s(__ldg(rec + r * NT));
-            Lam[r] = fault_update(msg, s, wr[r], C);
+            Lam[r] = fault_update(msg, fs.get(rec, r), wr[r], C);
         };
         auto any = [&](int r) {
             const int j = threadIdx.x + r * NT;
@@ -69,7 +64,7 @@ __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C,
                 Lam[r] = fault_update<float, DV>(msg, sl, deg, wr[r], C);
             }
         };
-        each_fault<VPT>(packed, fast, any);
+        each_fault<VPT>(fs.n, fast, any);
         __syncthreads();
     }
 }

@@ -323,6 +323,12 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     // packed slot records: [0, N) in messages, [N, 2 N) in bytes
     const bool rec_fits = g.msg_bytes / msg_size <= 65536, rec8_fits = g.msg_bytes <= 65536;
     std::vector<uint32_t> var_rec(4 * (size_t)N, 0u);
+    std::vector<uint8_t> packed32((N + 31) / 32, 0);
+    for (int q = 0; 32 * q + 32 <= N; ++q) {
+        packed32[q] = 1;
+        for (int j = 32 * q; j < 32 * q + 32; ++j)
+            if (var_deg[j] != 2 && var_deg[j] != 3) packed32[q] = 0;
+    }
     for (int j = 0; j < N; ++j) {
         const int32_t *sl = &var_slot[(size_t)j * DV];
         if (var_deg[j] == 2 || var_deg[j] == 3)
@@ -372,20 +378,21 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
 
     // one device arena for every graph array
     const size_t R1 = (size_t)d->prm.R + 1;
-    size_t off[9], o = 0;
-    const size_t sizes[9] = {(size_t)g.Mp, sizeof(int32_t) * N * DV, sizeof(uint32_t) * pad_mask.size(),
+    size_t off[10], o = 0;
+    const size_t sizes[10] = {(size_t)g.Mp, sizeof(int32_t) * N * DV, sizeof(uint32_t) * pad_mask.size(),
                              sizeof(int32_t) * N * DV, sizeof(float) * N, sizeof(float) * R1 * N,
                              sizeof(int32_t) * slot_edge.size(), sizeof(uint32_t) * var_rec.size(),
-                             sizeof(unsigned int) * 4};
-    for (int q = 0; q < 9; ++q) {
+                             packed32.size(), sizeof(unsigned int) * 4};
+    for (int q = 0; q < 10; ++q) {
         off[q] = o;
         o = align_up(o + sizes[q], 256);
     }
     QL_CUDA(cudaMalloc(&d->arena, o));
     char *base = static_cast<char *>(d->arena);
-    const void *src[8] = {chk_deg.data(), var_chk.data(), pad_mask.data(), var_slot.data(),
-                          w.data(), gamma, slot_edge.data(), var_rec.data()};
-    for (int q = 0; q < 8; ++q)
+    const void *src[9] = {chk_deg.data(), var_chk.data(), pad_mask.data(), var_slot.data(),
+                          w.data(), gamma, slot_edge.data(), var_rec.data(),
+                          packed32.data()};
+    for (int q = 0; q < 9; ++q)
         QL_CUDA(cudaMemcpy(base + off[q], src[q], sizes[q], cudaMemcpyHostToDevice));
     g.chk_deg = reinterpret_cast<const uint8_t *>(base + off[0]);
     g.var_chk = reinterpret_cast<const int32_t *>(base + off[1]);
@@ -397,7 +404,8 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     const uint2 *rec = reinterpret_cast<const uint2 *>(base + off[7]);
     g.var_rec = rec_fits ? rec : nullptr;
     g.var_rec8 = rec8_fits ? rec + N : nullptr;
-    d->counter = reinterpret_cast<unsigned int *>(base + off[8]);
+    g.packed32 = reinterpret_cast<const uint8_t *>(base + off[8]);
+    d->counter = reinterpret_cast<unsigned int *>(base + off[9]);
     QL_CUDA(cudaMemset(d->counter, 0, sizeof(unsigned int) * 4));
     return setup_tail(d, tab, ntab, tail_cut);
 }
@@ -463,8 +471,12 @@ int setup_baseline(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_
 int launch_persistent(const qldpc_decoder *d, const uint64_t *syn, int64_t B, DecodeOut out,
                       unsigned int *counter, ShotMap map, cudaStream_t st) {
     const bool tail = d->fk_tail != nullptr;
-    QL_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned int), st));
-    if (tail) QL_CUDA(cudaMemsetAsync(d->counter + 1, 0, 2 * sizeof(unsigned int), st));
+    if (counter == d->counter) {  // the tail's counters follow the work counter: one fill
+        QL_CUDA(cudaMemsetAsync(counter, 0, (tail ? 3 : 1) * sizeof(unsigned int), st));
+    } else {
+        QL_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned int), st));
+        if (tail) QL_CUDA(cudaMemsetAsync(d->counter + 1, 0, 2 * sizeof(unsigned int), st));
+    }
     const bool small = d->fk_small && B <= d->small_max;
     const FusedKernel *fk = small ? d->fk_small : d->fk;
     const int grid = (int)std::min<int64_t>(small ? d->small_grid : d->grid, B);

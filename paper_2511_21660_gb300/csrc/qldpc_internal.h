@@ -42,6 +42,7 @@ struct FusedGraph {
                               // messages; x = s0 | s1 << 16, y = s2 | degree << 16, degree 2
                               // with s2 = s0); nullptr when a slot does not fit 16 bits
     const uint2 *var_rec8;    // [N] the same with byte offsets; nullptr above 64 KB of messages
+    const uint8_t *packed32;  // [ceil(N/32)] 1: the group's 32 faults all have such a record
     const uint32_t *pad_mask; // [Mp/2][DC] binary16 only: 0xffff in each half of the
                               // pair's physical word p that holds a padding slot
     const float *w;           // [N] prior LLRs

@@ -149,20 +149,34 @@ struct Packed {
 
 // Fault slots of the warp (faults threadIdx.x + r NT) that take the packed-record path: the
 // slots r < n, n the number of leading slots whose 32 faults all exist and have degree 2 or 3.
-// Called by whole warps.
-template <typename MT, int NT, int VPT, int DV>
-__device__ __forceinline__ int packed_slots(const FusedGraph &g) {
-    if (!Packed<MT, NT * VPT>::table(g)) return 0;
-    int r = 0;
+// KEEP: their records stay in registers.  Set up by whole warps.
+template <typename MT, int NT, int VPT, bool KEEP = false>
+struct FaultSlots {
+    using P = Packed<MT, NT * VPT>;
+    int n;
+    uint2 kept[KEEP ? VPT : 1];
+    __device__ __forceinline__ void init(const FusedGraph &g) {
+        n = 0;
+        if (!P::table(g)) return;
+        const int groups = (g.N + 31) >> 5;
+        int r = 0;
 #pragma unroll 1
-    for (; r < VPT; ++r) {
-        const int j = threadIdx.x + r * NT;
-        int deg = 0;
-        if (j < g.N) deg = (int)((uint32_t)__ldg(g.var_slot + (size_t)j * DV) >> 24);
-        if (!__all_sync(FULL, deg == 2 || deg == 3)) break;
+        for (; r < VPT; ++r) {  // the vote makes the count uniform for the compiler
+            const int q = (int)(threadIdx.x >> 5) + r * (NT / 32);
+            if (!__all_sync(FULL, q < groups && __ldg(g.packed32 + q))) break;
+        }
+        n = r;
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int r = 0; r < VPT; ++r)
+                kept[r] = r < n ? __ldg(P::table(g) + threadIdx.x + r * NT) : make_uint2(0u, 0u);
+        }
     }
-    return r;
-}
+    __device__ __forceinline__ P get(const uint2 *rec, int r) const {  // rec: the thread's first
+        if constexpr (KEEP) return P(kept[r]);
+        else return P(__ldg(rec + r * NT));
+    }
+};
 
 // The per-fault loops: fast(r) for the packed slots and any(r) for the others.  (One loop body
 // with a branch per fault on its degree, a ballot and a bitmap store took 50 instructions a
@@ -202,9 +216,9 @@ __device__ __forceinline__ void each_fault(int packed, Fast fast, Any any) {
 //           (warm_mode 0) or w (warm_mode 1); nu(0) = lambda(0)
 // bb holds (1 - gamma_j) * lambda_j(0), rounded, which is the first product of
 // the memory update and is constant within a leg.
-template <typename MT, int NT, int VPT, int DV>
+template <typename MT, int NT, int VPT, int DV, typename FS>
 __device__ __forceinline__ void leg_init(const FusedGraph &g, const DevParams &p, int leg,
-                                         unsigned char *msg, int packed,
+                                         unsigned char *msg, const FS &fs,
                                          float (&Lam)[VPT], float (&bb)[VPT],
                                          float (&gg)[VPT]) {
     const float *grow = g.gamma + (size_t)leg * g.N + threadIdx.x;
@@ -224,7 +238,7 @@ __device__ __forceinline__ void leg_init(const FusedGraph &g, const DevParams &p
         for (int r = 0; r < VPT; ++r) bb[r] = canon(Lam[r]);
     }
     auto fast = [&](int r) {
-        const Packed<MT, NT * VPT> s(__ldg(rec + r * NT));
+        const Packed<MT, NT * VPT> s = fs.get(rec, r);
         const float lam0 = bb[r], gm = __ldg(grow + r * NT);
         Msg<MT>::st(msg, s.o0, lam0);
         Msg<MT>::st(msg, s.o1, lam0);
@@ -245,7 +259,7 @@ __device__ __forceinline__ void leg_init(const FusedGraph &g, const DevParams &p
             bb[r] = canon(__fmul_rn(__fsub_rn(1.0f, gm), lam0));
         }
     };
-    each_fault<VPT>(packed, fast, any);
+    each_fault<VPT>(fs.n, fast, any);
 }
 
 // The check rule's combination of two messages: the smaller magnitude with the product of
@@ -294,10 +308,21 @@ struct RowBits {
     uint32_t s0, s1, part;
 };
 
+// The rows of the thread that have padding slots; those slots get C, which the check pass
+// keeps there for good.  (Rows past the last check are never visited.)
 template <typename MT, int NT, int DC>
-__device__ __forceinline__ uint32_t partial_rows(const FusedGraph &g) {
+__device__ __forceinline__ uint32_t setup_rows(const FusedGraph &g, unsigned char *msg, float C) {
     uint32_t m = 0u;
     const bool half = sizeof(MT) == 2;
+    for (int i = threadIdx.x; i < g.Mp; i += NT) {
+        const int deg = g.chk_deg[i];
+        const int f = half ? swz<DC>(i >> 1) : swz<DC>(i);
+        for (int k = deg; k < DC; ++k) {
+            const int p = k ^ f;
+            const int off = half ? (((i >> 1) * DC + p) * 4 + (i & 1) * 2) : ((i * DC + p) * 4);
+            Msg<MT>::st(msg, off, C);
+        }
+    }
     const int rows = half ? (g.M + 1) >> 1 : g.M;
     for (int i = threadIdx.x, k = 0; i < rows; i += NT, ++k) {
         const bool full = half ? g.chk_deg[2 * i] == DC && g.chk_deg[2 * i + 1] == DC
@@ -494,9 +519,9 @@ __device__ __forceinline__ int check_of_slot(int off) {
 // The decision of a fault is the sign bit of its marginal (never -0, see fault_update), shifted
 // into a mask; the bitmap words and the parity flips follow for the warps that decided any.
 // Returns the thread's decided faults (bit VPT-1-r: fault threadIdx.x + r*NT has F_j = 1).
-template <typename MT, int NT, int VPT, int DC, int DV>
+template <typename MT, int NT, int VPT, int DC, int DV, typename FS>
 __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned char *msg, uint32_t *fw,
-                                           uint32_t *par, int packed, float (&Lam)[VPT],
+                                           uint32_t *par, const FS &fs, float (&Lam)[VPT],
                                            const float (&bb)[VPT], const float (&gg)[VPT],
                                            float C) {
     static_assert(VPT <= 32, "one decision bit per fault of the thread");
@@ -507,7 +532,7 @@ __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned cha
         dmask = __funnelshift_l(__float_as_uint(L), dmask, 1);  // dmask << 1 | sign(L)
     };
     auto fast = [&](int r) {
-        const Packed<MT, NT * VPT> s(__ldg(rec + r * NT));
+        const Packed<MT, NT * VPT> s = fs.get(rec, r);
         const float lam = __fadd_rn(bb[r], __fmul_rn(gg[r], Lam[r]));
         Lam[r] = fault_update(msg, s, lam, C);
         decide(Lam[r]);
@@ -524,7 +549,7 @@ __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned cha
         }
         decide(L);
     };
-    each_fault<VPT>(packed, fast, any);
+    each_fault<VPT>(fs.n, fast, any);
     __syncwarp();
     // bitmap words of the warp: fault slot r's 32 faults are word (wb + r NT) / 32
     uint32_t word = 0u;
@@ -629,21 +654,10 @@ __device__ __forceinline__ bool warp_same_solution(const uint32_t *fw, const uin
     return !__any_sync(FULL, diff != 0u);
 }
 
-// Padding slots of every check hold C for good (the check pass writes C back).
-template <typename MT, int NT, int DC>
-__device__ __forceinline__ void block_setup(const FusedGraph &g, unsigned char *msg, uint32_t *fw,
-                                            float C) {
+// Once a block: the bitmaps' words past the last fault stay zero.
+template <int NT>
+__device__ __forceinline__ void clear_bitmaps(const FusedGraph &g, uint32_t *fw) {
     for (int q = threadIdx.x; q < 2 * g.f_words; q += NT) fw[q] = 0u;  // fw and fb
-    for (int i = threadIdx.x; i < g.Mp; i += NT) {
-        const int deg = g.chk_deg[i];
-        const bool half = sizeof(MT) == 2;
-        const int f = half ? swz<DC>(i >> 1) : swz<DC>(i);
-        for (int k = deg; k < DC; ++k) {
-            const int p = k ^ f;
-            const int off = half ? (((i >> 1) * DC + p) * 4 + (i & 1) * 2) : ((i * DC + p) * 4);
-            Msg<MT>::st(msg, off, C);
-        }
-    }
 }
 
 template <int NT>
@@ -664,19 +678,20 @@ __device__ __forceinline__ void plain_bp(const FusedGraph &g, const DevParams &p
                                          const uint64_t *sy, unsigned char *msg, uint32_t *fw,
                                          uint32_t *sg, uint32_t *par,
                                          float (&Lam)[VPT], float (&bb)[VPT], float (&gg)[VPT]) {
-    block_setup<float, NT, DC>(g, msg, fw, p.clip);
+    clear_bitmaps<NT>(g, fw);
     load_syndrome<NT>(g, sy, sg);
-    const int packed = packed_slots<float, NT, VPT, DV>(g);
+    FaultSlots<float, NT, VPT> fs;
+    fs.init(g);
     RowBits rb;
-    rb.part = partial_rows<float, NT, DC>(g);
+    rb.part = setup_rows<float, NT, DC>(g, msg, p.clip);
     row_syndromes<float, NT>(g, sy, rb);
     __syncthreads();
-    leg_init<float, NT, VPT, DV>(g, p, 0, msg, packed, Lam, bb, gg);
+    leg_init<float, NT, VPT, DV>(g, p, 0, msg, fs, Lam, bb, gg);
     __syncthreads();
     for (int t = 0; t < iters; ++t) {
         check_pass<NT, DC>(g, reinterpret_cast<float *>(msg), sg, par, rb, p.clip);
         __syncthreads();
-        fault_pass<float, NT, VPT, DC, DV>(g, msg, fw, par, packed, Lam, bb, gg, p.clip);
+        fault_pass<float, NT, VPT, DC, DV>(g, msg, fw, par, fs, Lam, bb, gg, p.clip);
         __syncthreads();
     }
 }

@@ -46,6 +46,13 @@ struct ShotState {
     long long wacc[2];   // weight of the new solution, added up by its faults' threads
     long long best[2];   // weight of the kept solution (kNoWeight: none); copy in use: as wacc
 };
+// Shapes with registers to spare at their launch bounds' residency keep the slot records of
+// their faults there: it takes a load's latency out of every fault pass, which shows where
+// few warps hide it (8064 faults, 512 x 16, one block per SM: 1.68 -> 1.55 ms).  Giving up a
+// resident block for it does not pay (gross code, 256 x 11: 4 blocks 1.05, 3 blocks with the
+// records kept 1.15 ms).
+template <int NT, int VPT, int MINB>
+constexpr bool kKeep = (65536 / (NT * MINB) / 8 * 8) >= 5 * VPT + 31;
 constexpr long long kNoWeight = 0x7fffffffffffffffLL;
 
 // Relay on one shot: the leg schedule around the check and fault passes.  Per
@@ -61,12 +68,12 @@ constexpr long long kNoWeight = 0x7fffffffffffffffLL;
 // Tail continuation (TailCont): with tc.mode 1 a shot that reaches a leg boundary after
 // tc.cut iterations, with a next leg to run, may be suspended (its state saved in a
 // record, no outputs written); RESUME takes the shot of record st.rec up at its boundary.
-template <typename MT, int NT, int VPT, int DC, int DV, bool RESUME = false>
+template <typename MT, int NT, int VPT, int DC, int DV, bool RESUME = false, typename FS>
 __device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams &p,
                                             const uint64_t *__restrict__ syn, int syn_stride,
                                             int cor_stride, const DecodeOut &out,
                                             unsigned char *msg, uint32_t *fw, uint32_t *fb,
-                                            uint32_t *sg, uint32_t *par, ShotState &st, int packed, RowBits &rb,
+                                            uint32_t *sg, uint32_t *par, ShotState &st, const FS &fs, RowBits &rb,
                                             float (&Lam)[VPT], float (&bb)[VPT],
                                             float (&gg)[VPT], int &ab, const TailCont &tc) {
     const int tid = threadIdx.x;
@@ -108,7 +115,7 @@ __device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams
     uint32_t *pc = par;  // this iteration's parity words: the two buffers take turns
     bool fresh = false, done = false;
     for (;;) {
-        if (!done) leg_init<MT, NT, VPT, DV>(g, p, leg, msg, packed, Lam, bb, gg);
+        if (!done) leg_init<MT, NT, VPT, DV>(g, p, leg, msg, fs, Lam, bb, gg);
         // a long shot with a next leg to run is suspended if a record is free (the next
         // leg's initialisation is redone on resumption from the same state); thread 0
         // decides and takes the record, st.slot tells the block (-1: go on)
@@ -145,7 +152,7 @@ __device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams
         do {
             check_pass<NT, DC>(g, reinterpret_cast<MT *>(msg), sg, pc, rb, C);
             __syncthreads();
-            dm = fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, pc, packed, Lam, bb, gg, C);
+            dm = fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, pc, fs, Lam, bb, gg, C);
             __syncthreads();
             ++t;
             conv = warp_converged(pc, g.m_words);
@@ -195,11 +202,21 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode(FusedGraph g, DevParams
     uint32_t *fw, *fb, *sg, *par;
     smem_layout(g, smem_raw, fw, fb, sg, par);
     __shared__ ShotState st;
-    block_setup<MT, NT, DC>(g, msg, fw, p.clip);
+    // The resuming launch is queued as a programmatic dependent of the first one: its blocks
+    // may be placed while the first launch's last shots run, and wait here for its end.
+    if (RESUME)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    else
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int limit = RESUME ? (int)min(*tc.count, (unsigned int)tc.cap)
+                             : (map.order ? min(*map.count, B) : B);
+    if ((int)blockIdx.x >= limit) return;  // as many blocks as shots at most have work
+    clear_bitmaps<NT>(g, fw);
 
-    const int packed = packed_slots<MT, NT, VPT, DV>(g);
+    FaultSlots<MT, NT, VPT, kKeep<NT, VPT, MINB>> fs;
+    fs.init(g);
     RowBits rb;
-    rb.part = partial_rows<MT, NT, DC>(g);
+    rb.part = setup_rows<MT, NT, DC>(g, msg, p.clip);
 
     float Lam[VPT], bb[VPT], gg[VPT];
 #pragma unroll
@@ -207,8 +224,6 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode(FusedGraph g, DevParams
     int ab = 0;
     if (threadIdx.x < 2) st.wacc[threadIdx.x] = 0;
 
-    const int limit = RESUME ? (int)min(*tc.count, (unsigned int)tc.cap)
-                             : (map.order ? min(*map.count, B) : B);
     for (;;) {
         __syncthreads();  // the previous shot is done with shared memory and its state
         if (threadIdx.x == 0) {
@@ -223,7 +238,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode(FusedGraph g, DevParams
         __syncthreads();
         if (st.shot < 0) break;
         decode_shot<MT, NT, VPT, DC, DV, RESUME>(g, p, syn, map.syn_stride, map.cor_stride, out,
-                                                 msg, fw, fb, sg, par, st, packed, rb, Lam,
+                                                 msg, fw, fb, sg, par, st, fs, rb, Lam,
                                                  bb, gg, ab, tc);
     }
 }
@@ -244,7 +259,8 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode_multi(MultiTable tab,
     __shared__ ShotState st;
     __shared__ int s_code;
     int cur = -1;
-    int packed = 0;
+    FaultSlots<MT, NT, VPT> fs;
+    fs.n = 0;
     RowBits rb;
     rb.part = 0u;
 
@@ -281,14 +297,14 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode_multi(MultiTable tab,
         uint32_t *fw, *fb, *sg, *par;
             smem_layout(s_g, smem_raw, fw, fb, sg, par);
         if (code != cur) {
-            block_setup<MT, NT, DC>(s_g, msg, fw, s_p.clip);
-            packed = packed_slots<MT, NT, VPT, DV>(s_g);
-            rb.part = partial_rows<MT, NT, DC>(s_g);
+            clear_bitmaps<NT>(s_g, fw);
+            fs.init(s_g);
+            rb.part = setup_rows<MT, NT, DC>(s_g, msg, s_p.clip);
             cur = code;
             __syncthreads();
         }
         decode_shot<MT, NT, VPT, DC, DV>(s_g, s_p, syn, syn_stride, cor_stride, out, msg, fw, fb,
-                                         sg, par, st, packed, rb, Lam, bb, gg, ab,
+                                         sg, par, st, fs, rb, Lam, bb, gg, ab,
                                          TailCont{});
     }
 }
@@ -304,17 +320,18 @@ __global__ void __launch_bounds__(NT) fused_trace(FusedGraph g, DevParams p,
     smem_layout(g, smem_raw, fw, fb, sg, par);
     const int shot = blockIdx.x;
     const float C = p.clip;
-    block_setup<MT, NT, DC>(g, msg, fw, C);
+    clear_bitmaps<NT>(g, fw);
     load_syndrome<NT>(g, syn + (size_t)shot * g.syn_words, sg);
     float Lam[VPT], bb[VPT], gg[VPT];
 #pragma unroll
     for (int r = 0; r < VPT; ++r) Lam[r] = bb[r] = gg[r] = 0.0f;
-    const int packed = packed_slots<MT, NT, VPT, DV>(g);
+    FaultSlots<MT, NT, VPT> fs;
+    fs.init(g);
     RowBits rb;
-    rb.part = partial_rows<MT, NT, DC>(g);
+    rb.part = setup_rows<MT, NT, DC>(g, msg, p.clip);
     row_syndromes<MT, NT>(g, syn + (size_t)shot * g.syn_words, rb);
     __syncthreads();
-    leg_init<MT, NT, VPT, DV>(g, p, 0, msg, packed, Lam, bb, gg);
+    leg_init<MT, NT, VPT, DV>(g, p, 0, msg, fs, Lam, bb, gg);
     __syncthreads();
     const int nslots = g.msg_bytes / (int)sizeof(MT);
     for (int t = 0; t < T; ++t) {
@@ -327,7 +344,7 @@ __global__ void __launch_bounds__(NT) fused_trace(FusedGraph g, DevParams p,
                 if (e >= 0) mu[o * E + e] = Msg<MT>::ld(msg, s * (int)sizeof(MT));
             }
         __syncthreads();
-        fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, par, packed, Lam, bb, gg, C);
+        fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, par, fs, Lam, bb, gg, C);
         __syncthreads();
         if (marg) {
 #pragma unroll
@@ -351,6 +368,20 @@ template <typename MT, int NT, int VPT, int MINB, int DC, int DV, bool RESUME>
 cudaError_t launch_decode(dim3 grid, size_t smem, cudaStream_t st, const FusedGraph &g,
                           const DevParams &p, const uint64_t *syn, int B, DecodeOut out,
                           unsigned int *counter, ShotMap map, TailCont tc) {
+    if (RESUME) {  // without work it costs a call 1 us behind the first launch, not 5
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(NT);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, fused_decode<MT, NT, VPT, MINB, DC, DV, RESUME>, g, p, syn,
+                                  B, out, counter, map, tc);
+    }
     fused_decode<MT, NT, VPT, MINB, DC, DV, RESUME><<<grid, NT, smem, st>>>(g, p, syn, B, out,
                                                                             counter, map, tc);
     return cudaGetLastError();
