@@ -28,7 +28,7 @@ def _units():
     units = [("qldpc_api", "qldpc_api.cu", []), ("soft_api", "soft_api.cu", []),
              ("post_api", "post_api.cu", []), ("relay_baseline", "relay_baseline.cu", []),
              ("soft_dmem", "soft_dmem.cu", []), ("filtered_osd", "filtered_osd.cu", []),
-             ("cluster_decode", "cluster_decode.cu", [])]
+             ("cluster_decode", "cluster_decode.cu", []), ("relay_split", "relay_split.cu", [])]
     for f16, dc, dv in FUSED_FAMILIES:
         units.append((f"relay_fused_{'f16' if f16 else 'f32'}_{dc}_{dv}", "relay_fused.cu",
                       [f"-DQL_MSG_F16={f16}", f"-DQL_DC={dc}", f"-DQL_DV={dv}"]))

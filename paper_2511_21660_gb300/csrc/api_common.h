@@ -11,6 +11,7 @@
 
 #include "qldpc.h"
 #include "qldpc_internal.h"
+#include "relay_split.h"
 
 namespace qldpc {
 
@@ -81,6 +82,12 @@ struct qldpc_decoder {
     int tail_grid = 0;
     qldpc::TailCont tail{};  // mode 0 when off
     void *tail_arena = nullptr;
+    // resuming launch with a cluster of blocks per shot (nullptr: fk_tail resumes)
+    const qldpc::SplitKernel *fk_split = nullptr;
+    qldpc::SplitGraph split{};
+    size_t split_smem = 0;
+    int split_clusters = 0;
+    void *split_arena = nullptr;
     cudaStream_t stream = nullptr;  // internal stream of the host-buffer entry point
     void *stage = nullptr;
     int64_t stage_B = 0;

@@ -199,6 +199,15 @@ bool holds(const FusedKernel &k, int M, int N) {
     return (long long)k.threads * k.vpt >= N && 32LL * k.threads >= rows;
 }
 
+// Raises a kernel's limit of dynamic shared memory to `smem` (the limit belongs to the kernel,
+// which handles of several graphs share: it is never lowered).
+cudaError_t allow_smem(const void *fn, size_t smem) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= smem) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 // Small batches: with fewer shots than about twice the blocks that a wider shape keeps
 // resident, a shot's latency counts and the narrow shape's full residency does not.
 // Measured (us a launch, narrow / wide): gross code 100 shots 39.5 / 34.3, 608 101 / 87, 2400
@@ -212,8 +221,7 @@ int setup_small(qldpc_decoder *d) {
         return QLDPC_OK;
     }
     int bps = 0;
-    QL_CUDA(cudaFuncSetAttribute(d->fk_small->decode_fn,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem));
+    QL_CUDA(allow_smem(d->fk_small->decode_fn, d->smem));
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, d->fk_small->decode_fn,
                                                           d->fk_small->threads, d->smem));
     if (bps < 1) {
@@ -235,8 +243,7 @@ int setup_tail(qldpc_decoder *d, const FusedKernel *tab, int ntab, int tail_cut)
             (!d->fk_tail || tab[q].vpt < d->fk_tail->vpt))
             d->fk_tail = &tab[q];
     if (!d->fk_tail) return QLDPC_OK;  // no resuming shape holds the graph
-    QL_CUDA(cudaFuncSetAttribute(d->fk_tail->resume_fn,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem));
+    QL_CUDA(allow_smem(d->fk_tail->resume_fn, d->smem));
     int bps = 0;
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, d->fk_tail->resume_fn,
                                                           d->fk_tail->threads, d->smem));
@@ -254,6 +261,134 @@ int setup_tail(qldpc_decoder *d, const FusedKernel *tab, int ntab, int tail_cut)
     tc.lam = reinterpret_cast<float *>(static_cast<char *>(d->tail_arena) + rec_bytes);
     tc.count = d->counter + 1;
     tc.mode = 1;
+    return QLDPC_OK;
+}
+
+// The resuming launch that spreads a shot over a cluster of kSplit blocks (relay_split.cu): the
+// checks cut into contiguous ranges where the fewest faults reach across, near equal sizes;
+// each fault with its first check.  Rows of up to 8 slots and faults of degree up to 4 that
+// fit a compiled shape; otherwise one block resumes a shot.
+int setup_split(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx) {
+    const FusedGraph &fg = d->fg;
+    const int M = d->M, N = d->N, DC = d->fk->dc, DV = d->fk->dv, half = d->msg_fp16;
+    if (DC != 8 || DV != 4 || M < 64 * kSplit) return QLDPC_OK;
+    SplitGraph &g = d->split;
+    // checks of each fault, ascending, with the edge's place in its row
+    std::vector<int> deg(N, 0), chk((size_t)N * DV), place((size_t)N * DV);
+    for (int i = 0; i < M; ++i)
+        for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
+            const size_t q = (size_t)col_idx[e] * DV + deg[col_idx[e]]++;
+            chk[q] = i;
+            place[q] = e - row_ptr[i];
+        }
+    std::vector<int> across(M + 2, 0);  // faults with checks on both sides of a cut before i
+    for (int j = 0; j < N; ++j)
+        if (deg[j] > 1) {
+            ++across[chk[(size_t)j * DV] + 1];
+            --across[chk[(size_t)j * DV + deg[j] - 1] + 1];
+        }
+    for (int i = 1; i <= M; ++i) across[i] += across[i - 1];
+    g.row0[0] = 0;
+    g.row0[kSplit] = M;
+    for (int b = 1; b < kSplit; ++b) {
+        const int at = (int)((long long)M * b / kSplit) & ~1, reach = M / (4 * kSplit);
+        int best = at;
+        for (int c = std::max(at - reach, 2) & ~1; c <= at + reach; c += 2)
+            if (across[c] < across[best] ||
+                (across[c] == across[best] && std::abs(c - at) < std::abs(best - at)))
+                best = c;
+        g.row0[b] = best;
+    }
+    int rows = 0;
+    std::vector<int> block(M);
+    for (int b = 0; b < kSplit; ++b) {
+        const int r = g.row0[b + 1] - g.row0[b];
+        rows = std::max(rows, (r + 1) & ~1);
+        for (int i = g.row0[b]; i < g.row0[b + 1]; ++i) block[i] = b;
+    }
+    std::vector<int> home(N, 0);
+    size_t held[kSplit] = {}, most = 0;
+    for (int j = 0; j < N; ++j) {
+        if (deg[j] > 0) home[j] = block[chk[(size_t)j * DV]];
+        most = std::max(most, ++held[home[j]]);
+    }
+    const SplitKernel *tab = nullptr;
+    int ntab = 0;
+    split_table(&tab, &ntab);
+    const SplitKernel *k = nullptr;
+    for (int q = 0; q < ntab && !k; ++q)
+        if (tab[q].msg_fp16 == half && d->dv_max <= tab[q].dv &&
+            (size_t)tab[q].threads * tab[q].vpt >= most)
+            k = &tab[q];
+    if (!k) return QLDPC_OK;
+
+    // message rows as in setup_fused, by the row's index in its block
+    auto swz = [](int x) { return (x >> 2) & 7; };
+    auto off = [&](int r, int p) {
+        return half ? ((r >> 1) * DC + (p ^ swz(r >> 1))) * 4 + (r & 1) * 2
+                    : (r * DC + (p ^ swz(r))) * 4;
+    };
+    const int msg_size = half ? 2 : 4;
+    g.N = N;
+    g.cor_words = fg.cor_words;
+    g.min_deg = fg.min_deg;
+    g.msg_bytes = rows * DC * msg_size;
+    g.rows = rows;
+    g.pad_stride = rows / 2 * DC;
+    const size_t cap = (size_t)k->threads * k->vpt;
+    const size_t s_fault = align_up(sizeof(int32_t) * kSplit * cap, 256);
+    const size_t s_slots = align_up(4 * sizeof(uint32_t) * kSplit * cap, 256);
+    std::vector<unsigned char> image(s_fault + s_slots + sizeof(uint32_t) * kSplit * g.pad_stride);
+    int32_t *fault = reinterpret_cast<int32_t *>(image.data());
+    uint32_t *slots = reinterpret_cast<uint32_t *>(image.data() + s_fault);
+    uint32_t *pad = reinterpret_cast<uint32_t *>(image.data() + s_fault + s_slots);
+    std::fill(fault, fault + kSplit * cap, -1);
+    std::fill(slots, slots + 4 * kSplit * cap, kNoSlot);
+    size_t next[kSplit] = {};
+    for (int j = 0; j < N; ++j) {
+        const size_t q = home[j] * cap + next[home[j]]++;
+        fault[q] = j;
+        for (int e = 0; e < deg[j]; ++e) {
+            const int i = chk[(size_t)j * DV + e], c = block[i];
+            slots[4 * q + e] = ((uint32_t)c << 24) |
+                               (uint32_t)off(i - g.row0[c], place[(size_t)j * DV + e]);
+        }
+    }
+    for (int b = 0; half && b < kSplit; ++b)
+        for (int r = 0; r < rows; ++r) {
+            const int i = g.row0[b] + r;
+            const int d = i < g.row0[b + 1] ? row_ptr[i + 1] - row_ptr[i] : 0;
+            for (int q = d; q < DC; ++q)
+                pad[(size_t)b * g.pad_stride + (r >> 1) * DC + (q ^ swz(r >> 1))] |=
+                    (r & 1) ? 0xffff0000u : 0x0000ffffu;
+        }
+    const size_t smem = split_smem_bytes(g);
+    QL_CUDA(allow_smem(k->fn, smem));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kSplit);
+    cfg.blockDim = dim3(k->threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kSplit;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    QL_CUDA(cudaOccupancyMaxActiveClusters(&clusters, k->fn, &cfg));
+    if (clusters < 1) return QLDPC_OK;
+    QL_CUDA(cudaMalloc(&d->split_arena, image.size()));
+    char *base = static_cast<char *>(d->split_arena);
+    QL_CUDA(cudaMemcpy(base, image.data(), image.size(), cudaMemcpyHostToDevice));
+    g.chk_deg = fg.chk_deg;
+    g.fault = reinterpret_cast<const int32_t *>(base);
+    g.slots = reinterpret_cast<const uint4 *>(base + s_fault);
+    g.pad_mask = reinterpret_cast<const uint32_t *>(base + s_fault + s_slots);
+    g.w = fg.w;
+    g.gamma = fg.gamma;
+    d->fk_split = k;
+    d->split_smem = smem;
+    d->split_clusters = std::min(clusters, d->tail.cap);
     return QLDPC_OK;
 }
 
@@ -358,16 +493,14 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     if (state > (size_t)optin)
         return fail(QLDPC_ERR_UNSUPPORTED, "per-shot state needs %zu B of shared memory, above %d",
                     state, optin);
-    QL_CUDA(cudaFuncSetAttribute(d->fk->decode_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)d->smem));
+    QL_CUDA(allow_smem(d->fk->decode_fn, d->smem));
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->blocks_per_sm, d->fk->decode_fn,
                                                           d->fk->threads, d->smem));
     if (d->blocks_per_sm < 1)
         return fail(QLDPC_ERR_UNSUPPORTED, "the decode kernel cannot be resident on an SM");
     if (d->fk_trace) {
         d->trace_smem = d->smem;
-        QL_CUDA(cudaFuncSetAttribute(d->fk_trace->trace_fn,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d->smem));
+        QL_CUDA(allow_smem(d->fk_trace->trace_fn, d->smem));
     }
     d->block_threads = d->fk->threads;
     d->grid = d->num_sms * d->blocks_per_sm;
@@ -407,7 +540,9 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
     g.packed32 = reinterpret_cast<const uint8_t *>(base + off[8]);
     d->counter = reinterpret_cast<unsigned int *>(base + off[9]);
     QL_CUDA(cudaMemset(d->counter, 0, sizeof(unsigned int) * 4));
-    return setup_tail(d, tab, ntab, tail_cut);
+    rc = setup_tail(d, tab, ntab, tail_cut);
+    if (rc == QLDPC_OK && d->fk_tail) rc = setup_split(d, row_ptr, col_idx);
+    return rc;
 }
 
 int setup_baseline(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx,
@@ -481,11 +616,21 @@ int launch_persistent(const qldpc_decoder *d, const uint64_t *syn, int64_t B, De
     const FusedKernel *fk = small ? d->fk_small : d->fk;
     const int grid = (int)std::min<int64_t>(small ? d->small_grid : d->grid, B);
     QL_CUDA(fk->launch_decode(dim3(grid), d->smem, st, d->fg, d->prm, syn, (int)B, out, counter,
-                              map, d->tail));
-    if (tail)
+                              map, d->tail, 0));
+    if (!tail) return QLDPC_OK;
+    // With a split launch, up to split_clusters records go to it (a cluster of blocks each, all
+    // resident) and more to the one-block launch: gross code at p = 0.02, 17 records 30.1 ms
+    // with one block a shot, 24.0 split; 42 31.6 / 28.3; about 130 39 / 69.  A small batch, which
+    // cannot have many, leaves the one-block launch out.
+    const bool one_block = !d->fk_split || B > 8LL * d->split_clusters;
+    if (d->fk_split)
+        QL_CUDA(d->fk_split->launch(d->split_clusters, d->split_smem, st, d->split, d->prm, syn, out,
+                                    d->counter + 2, map, d->tail,
+                                    one_block ? d->split_clusters : d->tail.cap));
+    if (one_block)
         QL_CUDA(d->fk_tail->launch_resume(dim3(std::min(d->tail_grid, d->tail.cap)), d->smem, st,
                                           d->fg, d->prm, syn, (int)B, out, d->counter + 2, map,
-                                          d->tail));
+                                          d->tail, d->fk_split ? d->split_clusters : 0));
     return QLDPC_OK;
 }
 
@@ -768,8 +913,7 @@ int qldpc_decode_batch_multi(qldpc_decoder *const *decoders, int32_t n_codes,
         tab.p[c] = decoders[c]->prm;
         smem = std::max(smem, decoders[c]->smem);
     }
-    QL_CUDA(cudaFuncSetAttribute(fk->multi_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
+    QL_CUDA(allow_smem(fk->multi_fn, smem));
     int bps = 0;
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fk->multi_fn, fk->threads, smem));
     if (bps < 1) return fail(QLDPC_ERR_UNSUPPORTED, "mixed-batch kernel cannot be resident");
@@ -932,6 +1076,7 @@ void qldpc_destroy(qldpc_decoder *d) {
     }
     if (d->arena) cudaFree(d->arena);  // cudaFree waits for work that may still use it
     if (d->tail_arena) cudaFree(d->tail_arena);
+    if (d->split_arena) cudaFree(d->split_arena);
     if (d->stage) cudaFree(d->stage);
     delete d;
 }

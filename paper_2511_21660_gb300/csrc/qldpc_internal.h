@@ -123,11 +123,11 @@ struct FusedKernel {
     const void *decode_fn;   // __global__ symbol of the decode kernel
     cudaError_t (*launch_decode)(dim3 grid, size_t smem, cudaStream_t st, const FusedGraph &g,
                                  const DevParams &p, const uint64_t *syn, int B, DecodeOut out,
-                                 unsigned int *counter, ShotMap map, TailCont tc);
+                                 unsigned int *counter, ShotMap map, TailCont tc, int least);
     const void *resume_fn;   // __global__ symbol of the resuming instance (nullptr if none)
     cudaError_t (*launch_resume)(dim3 grid, size_t smem, cudaStream_t st, const FusedGraph &g,
                                  const DevParams &p, const uint64_t *syn, int B, DecodeOut out,
-                                 unsigned int *counter, ShotMap map, TailCont tc);
+                                 unsigned int *counter, ShotMap map, TailCont tc, int least);
     const void *multi_fn;    // __global__ symbol of the mixed-batch kernel
     cudaError_t (*launch_multi)(dim3 grid, size_t smem, cudaStream_t st, const MultiTable &tab,
                                 const int32_t *code_of_shot, const uint64_t *syn,

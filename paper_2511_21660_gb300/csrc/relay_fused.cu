@@ -52,7 +52,7 @@ struct ShotState {
 // resident block for it does not pay (gross code, 256 x 11: 4 blocks 1.05, 3 blocks with the
 // records kept 1.15 ms).
 template <int NT, int VPT, int MINB>
-constexpr bool kKeep = (65536 / (NT * MINB) / 8 * 8) >= 5 * VPT + 31;
+constexpr bool kKeep = QL_DC == 8 && (65536 / (NT * MINB) / 8 * 8) >= 5 * VPT + 31;
 constexpr long long kNoWeight = 0x7fffffffffffffffLL;
 
 // Relay on one shot: the leg schedule around the check and fault passes.  Per
@@ -191,12 +191,12 @@ __device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams
 // One block per shot at a time; shots come from a global counter (through the shot
 // map's index list when it has one).
 // RESUME: the second launch of the tail continuation; shots come from the records of the
-// first launch (counter then numbers the records taken).
+// first launch (counter then numbers the records taken), when there are more than `least`.
 template <typename MT, int NT, int VPT, int MINB, int DC, int DV, bool RESUME = false>
 __global__ void __launch_bounds__(NT, MINB) fused_decode(FusedGraph g, DevParams p,
                                                    const uint64_t *__restrict__ syn, int B,
                                                    DecodeOut out, unsigned int *counter,
-                                                   ShotMap map, TailCont tc) {
+                                                   ShotMap map, TailCont tc, int least) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *msg = smem_raw;
     uint32_t *fw, *fb, *sg, *par;
@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode(FusedGraph g, DevParams
     const int limit = RESUME ? (int)min(*tc.count, (unsigned int)tc.cap)
                              : (map.order ? min(*map.count, B) : B);
     if ((int)blockIdx.x >= limit) return;  // as many blocks as shots at most have work
+    if (RESUME && limit <= least) return;  // the split launch has taken them
     clear_bitmaps<NT>(g, fw);
 
     FaultSlots<MT, NT, VPT, kKeep<NT, VPT, MINB>> fs;
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(NT) fused_trace(FusedGraph g, DevParams p,
 template <typename MT, int NT, int VPT, int MINB, int DC, int DV, bool RESUME>
 cudaError_t launch_decode(dim3 grid, size_t smem, cudaStream_t st, const FusedGraph &g,
                           const DevParams &p, const uint64_t *syn, int B, DecodeOut out,
-                          unsigned int *counter, ShotMap map, TailCont tc) {
+                          unsigned int *counter, ShotMap map, TailCont tc, int least) {
     if (RESUME) {  // without work it costs a call 1 us behind the first launch, not 5
         cudaLaunchAttribute attr{};
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -380,10 +381,10 @@ cudaError_t launch_decode(dim3 grid, size_t smem, cudaStream_t st, const FusedGr
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, fused_decode<MT, NT, VPT, MINB, DC, DV, RESUME>, g, p, syn,
-                                  B, out, counter, map, tc);
+                                  B, out, counter, map, tc, least);
     }
     fused_decode<MT, NT, VPT, MINB, DC, DV, RESUME><<<grid, NT, smem, st>>>(g, p, syn, B, out,
-                                                                            counter, map, tc);
+                                                                            counter, map, tc, least);
     return cudaGetLastError();
 }
 

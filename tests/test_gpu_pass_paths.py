@@ -123,3 +123,24 @@ def test_few_faults_with_many_checks_take_a_wide_enough_block():
         ref = relay_decode(P.row_ptr, P.col_idx, P.p, gam, sig, RelayParams(**cfg),
                            precision=PREC[prec])
         assert_same_decisions(got, ref, f"tall/{PREC[prec]}")
+
+
+def test_handles_that_share_a_shape_keep_their_shared_memory():
+    """Two graphs on one compiled shape, the one with more shared memory created first."""
+    big, small = (phenomenological_dem(BB288, t, 0.003) for t in (18, 16))
+    for P in (big, small):
+        P.meta["code"] = "bb288"
+    cfg = RelayConfig(legs_after_first=20, stop_after_solutions=2)
+    sig = shots(big, 800, 4)[1]
+    gam = gamma_for(big, R=20)
+    want = gpu_decode(big, gam, sig, cfg)
+    first = RelayDecoder(big.row_ptr, big.col_idx, big.p, gam, cfg)
+    second = RelayDecoder(small.row_ptr, small.col_idx, small.p, gamma_for(small, R=20), cfg)
+    assert first.info.block_threads == second.info.block_threads
+    assert first.info.smem_bytes > second.info.smem_bytes > 48 * 1024
+    got = first.decode(torch.from_numpy(pack_bits(sig).view(np.int64)).cuda())
+    torch.cuda.synchronize()
+    for a, b in zip(got[1:], want[1:4]):                 # legs, converged, iterations
+        assert np.array_equal(a.cpu().numpy(), b)
+    first.close()
+    second.close()
