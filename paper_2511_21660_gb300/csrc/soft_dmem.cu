@@ -39,20 +39,32 @@ constexpr unsigned FULL = 0xffffffffu;
 
 template <typename T>
 struct RM;
-// float32: tanh(x/2) and atanh from the hardware exponential and logarithm and an
-// approximate division (absolute errors of a few 1e-7, far inside the float32 path's
-// tolerance against the FP64 oracle); FP64 keeps the library functions.
+// float32: tanh(x/2) and atanh from the hardware exponential, reciprocal and logarithm
+// (absolute errors of a few 1e-7, far inside the float32 path's tolerance against the FP64
+// oracle); FP64 keeps the library functions.  The flush-to-zero forms are one instruction each:
+// the others add scaling of subnormal operands and results around it, which cannot matter
+// here (1 + e^x >= 1, and the logarithm's argument lies in [2^-24, 2^24]).
 template <>
 struct RM<float> {
+    static __device__ __forceinline__ float rcp(float x) {
+        float y;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+        return y;
+    }
     // tanh(x/2) = 1 - 2/(1 + e^x); e^x = inf gives 1 and e^x = 0 gives -1
     static __device__ __forceinline__ float tanh_half(float x) {
-        return 1.0f - __fdividef(2.0f, 1.0f + __expf(x));
+        float e;
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * 1.44269504088896341f));
+        return 1.0f - 2.0f * rcp(1.0f + e);
     }
-    // atanh(x) = log((1 + x)/(1 - x)) / 2, for |x| <= 1 - 2^-23 (products are clamped)
-    static __device__ __forceinline__ float atanh_(float x) {
-        return 0.5f * __logf(__fdividef(1.0f + x, 1.0f - x));
+    // 2 atanh(x) / kUnit = log2((1 + x)/(1 - x)), for |x| <= 1 - 2^-23 (products are clamped)
+    static constexpr float kUnit = 0.693147180559945309f;
+    static __device__ __forceinline__ float two_atanh(float x) {
+        float y;
+        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((1.0f + x) * rcp(1.0f - x)));
+        return y;
     }
-    static __device__ __forceinline__ float div(float x, float y) { return __fdividef(x, y); }
+    static __device__ __forceinline__ float div(float x, float y) { return x * rcp(y); }
     static __device__ __forceinline__ float softplus(float x) {
         return x > 0.0f ? x + log1pf(expf(-x)) : log1pf(expf(x));
     }
@@ -63,7 +75,8 @@ struct RM<float> {
 template <>
 struct RM<double> {
     static __device__ __forceinline__ double tanh_half(double x) { return tanh(x / 2.0); }
-    static __device__ __forceinline__ double atanh_(double x) { return atanh(x); }
+    static constexpr double kUnit = 2.0;
+    static __device__ __forceinline__ double two_atanh(double x) { return atanh(x); }
     static __device__ __forceinline__ double div(double x, double y) { return x / y; }
     static __device__ __forceinline__ double softplus(double x) {
         return x > 0.0 ? x + log1p(exp(-x)) : log1p(exp(x));
@@ -243,9 +256,9 @@ __device__ __forceinline__ void soft_iteration(const SoftArgs<T> &a, const uint6
         row_tanh<T, DCM>(v, d, tau);
         if (tau_out) store_row<T, DCM>(tau_out + e0, i, d, tau);
         row_products<T, DCM>(tau, d, a.eps, P, cl);
-        const T s = bit_of(sy, i) ? T(-2) : T(2);
+        const T c = at * (bit_of(sy, i) ? -RM<T>::kUnit : RM<T>::kUnit);
 #pragma unroll
-        for (int k = 0; k < DCM; ++k) v[k] = k < d ? at * s * RM<T>::atanh_(P[k]) : T(0);
+        for (int k = 0; k < DCM; ++k) v[k] = k < d ? c * RM<T>::two_atanh(P[k]) : T(0);
         store_row<T, DCM>(nu + e0, i, d, v);
     }
     __syncthreads();
@@ -472,13 +485,14 @@ __global__ void __launch_bounds__(SOFT_BWD_THREADS, padded_rows<T, DCM>() ? SOFT
                 row_products<T, DCM>(tau, d, a.eps, P, cl);
                 load_row<T, DCM>(nb + e0, i, d, mbv);
                 const T s2 = bit_of(sy, i) ? T(-2) : T(2);
+                const T su = bit_of(sy, i) ? -RM<T>::kUnit : RM<T>::kUnit, as2 = at * s2;
 #pragma unroll
                 for (int k = 0; k < DCM; ++k) {
                     Pb[k] = 0;
                     if (k < d) {
                         const T mb = mbv[k];
-                        apart += mb * s2 * RM<T>::atanh_(P[k]);
-                        if (!cl[k]) Pb[k] = RM<T>::div(mb * at * s2, T(1) - P[k] * P[k]);
+                        apart += mb * su * RM<T>::two_atanh(P[k]);
+                        if (!cl[k]) Pb[k] = RM<T>::div(mb * as2, T(1) - P[k] * P[k]);
                     }
                 }
                 // tau_bar_k = sum_{m != k} Pb_m prod_{l != m, k} tau_l in O(d), without
@@ -518,14 +532,36 @@ __global__ void __launch_bounds__(SOFT_BWD_THREADS, padded_rows<T, DCM>() ? SOFT
     for (int t = threadIdx.x; t < a.T_it; t += NT) a.shot_ga[(size_t)b * a.T_it + t] = as[t];
 }
 
-// out[c] = scale * upstream * sum_b in[b][c], summed over b in order.
+// out[c] = scale * upstream * sum_b in[b][c], in a fixed order: 32 columns a block, warp y adds
+// the rows y, y + 32, ... and the 32 partial sums are added in pairs.  One thread a column
+// over all rows was a chain of B dependent additions behind its loads, on 22 blocks for the
+// 2736 gamma columns and on one for the loss and the alphas: REDUCE_BEFORE -> REDUCE_AFTER us for the three sums
+// of a step at 2048 shots.
+constexpr int kSumRows = 32;
 template <typename T>
-__global__ void reduce_shots(const T *in, int B, int n, T scale, const T *upstream, T *out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
+__global__ void __launch_bounds__(32 * kSumRows) reduce_shots(const T *in, int B, int n, T scale,
+                                                              const T *upstream, T *out) {
+    __shared__ T part[kSumRows][33];
+    const int x = threadIdx.x, y = threadIdx.y, c = blockIdx.x * 32 + x;
     T s = 0;
-    for (int b = 0; b < B; ++b) s += in[(size_t)b * n + c];
-    out[c] = s * scale * (upstream ? *upstream : T(1));
+    if (c < n) {
+#pragma unroll 8
+        for (int b = y; b < B; b += kSumRows) s += in[(size_t)b * n + c];
+    }
+    part[y][x] = s;
+    __syncthreads();
+    for (int h = kSumRows / 2; h > 0; h >>= 1) {
+        if (y < h) part[y][x] += part[y + h][x];
+        __syncthreads();
+    }
+    if (y == 0 && c < n) out[c] = part[0][x] * scale * (upstream ? *upstream : T(1));
+}
+
+template <typename T>
+cudaError_t sum_shots(const T *in, int B, int n, T scale, const T *upstream, T *out,
+                      cudaStream_t st) {
+    reduce_shots<T><<<(n + 31) / 32, dim3(32, kSumRows), 0, st>>>(in, B, n, scale, upstream, out);
+    return cudaGetLastError();
 }
 
 template <typename T>
@@ -564,9 +600,7 @@ cudaError_t run_forward_t(const SoftLaunch &L, cudaStream_t st) {
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const T scale = T(1) / ((T)L.B * (T)L.g.N);
-    reduce_shots<T><<<1, 32, 0, st>>>(a.shot_loss, L.B, 1, scale, nullptr,
-                                      static_cast<T *>(L.loss));
-    return cudaGetLastError();
+    return sum_shots<T>(a.shot_loss, L.B, 1, scale, nullptr, static_cast<T *>(L.loss), st);
 }
 
 template <typename T, int DCM>
@@ -599,11 +633,9 @@ cudaError_t run_backward_t(const SoftLaunch &L, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const T scale = T(1) / ((T)L.B * (T)L.g.N);
     const T *up = static_cast<const T *>(L.upstream);
-    reduce_shots<T><<<(L.g.N + 127) / 128, 128, 0, st>>>(a.shot_gg, L.B, L.g.N, scale, up,
-                                                         static_cast<T *>(L.grad_gamma));
-    reduce_shots<T><<<(L.T_it + 127) / 128, 128, 0, st>>>(a.shot_ga, L.B, L.T_it, scale, up,
-                                                          static_cast<T *>(L.grad_alpha));
-    return cudaGetLastError();
+    e = sum_shots<T>(a.shot_gg, L.B, L.g.N, scale, up, static_cast<T *>(L.grad_gamma), st);
+    if (e != cudaSuccess) return e;
+    return sum_shots<T>(a.shot_ga, L.B, L.T_it, scale, up, static_cast<T *>(L.grad_alpha), st);
 }
 
 }  // namespace
