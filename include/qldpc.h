@@ -67,9 +67,10 @@ typedef struct {
                                      Copied at create time; finite values required.        */
     int32_t tail_cut_iters;       /* tail continuation of the fused kernel: a shot that has
                                      run this many iterations when a leg ends, with a next
-                                     leg to run, is handed to a second launch with one
-                                     1024-thread block per SM (same results, lower latency
-                                     for the few very long shots).  0: T_1 + 8 T_r;
+                                     leg to run, is handed to a second launch: a cluster of
+                                     blocks per shot when few are left, else one 1024-thread
+                                     block per SM (same results, lower latency for the few
+                                     very long shots).  0: T_1 + 8 T_r;
                                      < 0: off                                              */
 } qldpc_relay_params;
 
@@ -90,7 +91,7 @@ typedef struct {
     int32_t correction_words;     /* ceil(N/64): uint64 words per correction                 */
     int32_t tail_cut_iters;       /* iterations before a shot may move to the second launch
                                      (-1: no tail continuation)                             */
-    int32_t tail_block_threads;   /* block size of the second launch                        */
+    int32_t tail_block_threads;   /* block size of the second launch with a block per shot   */
     int32_t tail_records;         /* shots the second launch can take per call; later long
                                      shots finish in the first launch                       */
 } qldpc_info;

@@ -288,6 +288,24 @@ __device__ __forceinline__ void excluded(const V (&a)[n], V rest, V (&o)[n]) {
     if constexpr (n == 2) {
         o[0] = minsign(a[1], rest);
         o[1] = minsign(a[0], rest);
+    } else if constexpr (n == 32) {  // by groups of 8: the whole tree's values would spill
+        V q[4], e[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            q[h] = a[8 * h];
+#pragma unroll
+            for (int k = 1; k < 8; ++k) q[h] = minsign(q[h], a[8 * h + k]);
+        }
+        excluded<4>(q, rest, e);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            V x[8], y[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = a[8 * h + k];
+            excluded<8>(x, e[h], y);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) o[8 * h + k] = y[k];
+        }
     } else {
         V p[n / 2], e[n / 2];
 #pragma unroll
@@ -632,7 +650,7 @@ __device__ __forceinline__ void smem_layout(const FusedGraph &g, unsigned char *
 // Plain min-sum BP (paper Sec. 2.3, "Belief propagation decoding"): DMem-BP with every
 // gamma_j = 0, which the graph's gamma row (all zeros) provides, from the priors, for
 // `iters` iterations without early exit; the marginals end in Lam.  Re-stages the
-// padding slots and priors first (callers reuse the message area between shots).
+// padding slots first (callers reuse the message area between shots).
 // Called by every thread of the block.
 template <int NT, int VPT, int DC, int DV>
 __device__ __forceinline__ void plain_bp(const FusedGraph &g, const DevParams &p, int iters,

@@ -11,8 +11,9 @@
 //     consecutive checks fall into distinct banks;
 //   * the per-fault state (Lambda_j, (1-gamma_j) lambda_j(0), gamma_j) lives in
 //     registers: fault j belongs to thread j mod NT for the whole shot;
-//   * decisions F_j = [Lambda_j < 0] are packed by warp ballots into a bitmap, and
-//     the syndrome H F is accumulated by the (few) faults with F_j = 1.
+//   * decisions F_j = [Lambda_j < 0] are sign bits; the warps that decided any fault
+//     write them to a bitmap and flip their checks in sigma + H F, which is 0 when
+//     the decision explains the syndrome.
 // All float arithmetic rounds every + and * separately (__fadd_rn/__fmul_rn), in
 // the same order as the single-precision oracle, so results are bit-identical.
 //
