@@ -605,7 +605,7 @@ int setup_baseline(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_
 // shape) finishes them.  Both on `st`, so the pair can be captured in a CUDA graph.
 int launch_persistent(const qldpc_decoder *d, const uint64_t *syn, int64_t B, DecodeOut out,
                       unsigned int *counter, ShotMap map, cudaStream_t st) {
-    const bool tail = d->fk_tail != nullptr;
+    const bool tail = d->fk_tail && d->prm.R > 0;  // a first leg alone has no boundary to stop at
     if (counter == d->counter) {  // the tail's counters follow the work counter: one fill
         QL_CUDA(cudaMemsetAsync(counter, 0, (tail ? 3 : 1) * sizeof(unsigned int), st));
     } else {

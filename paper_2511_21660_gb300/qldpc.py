@@ -358,11 +358,11 @@ class RelayDecoder:
 
     def outputs(self, B: int):
         import torch
-        dev = torch.device("cuda", self.device)
-        return (torch.empty((B, self.correction_words), dtype=torch.int64, device=dev),
-                torch.empty(B, dtype=torch.int32, device=dev),
-                torch.empty(B, dtype=torch.uint8, device=dev),
-                torch.empty(B, dtype=torch.int32, device=dev))
+        empty, dev = torch.empty, torch.device("cuda", self.device)
+        return (empty((B, self.correction_words), dtype=torch.int64, device=dev),
+                empty(B, dtype=torch.int32, device=dev),
+                empty(B, dtype=torch.uint8, device=dev),
+                empty(B, dtype=torch.int32, device=dev))
 
     def decode(self, syndromes, out=None, stream=None):
         """syndromes: int64 CUDA tensor [B, ceil(M/64)] (bit-packed uint64 words).
@@ -374,12 +374,14 @@ class RelayDecoder:
         if not syndromes.is_cuda or syndromes.dim() != 2 or \
                 syndromes.shape[1] != self.syndrome_words or not syndromes.is_contiguous():
             raise ValueError("syndromes must be a contiguous CUDA tensor [B, ceil(M/64)]")
+        import torch
         B = syndromes.shape[0]
         cor, legs, conv, iters = out if out is not None else self.outputs(B)
-        qldpc_decode_batch(self.handle, ctypes.c_void_p(syndromes.data_ptr()), B,
-                           ctypes.c_void_p(cor.data_ptr()), ctypes.c_void_p(legs.data_ptr()),
-                           ctypes.c_void_p(conv.data_ptr()), ctypes.c_void_p(iters.data_ptr()),
-                           self._stream_ptr(stream))
+        s = stream if stream is not None else torch.cuda.current_stream()
+        # addresses as plain integers: a small batch's call is bound by this marshalling
+        _check(_LIB.qldpc_decode_batch(self.handle, syndromes.data_ptr(), B, cor.data_ptr(),
+                                       legs.data_ptr(), conv.data_ptr(), iters.data_ptr(),
+                                       s.cuda_stream), "qldpc_decode_batch")
         return cor, legs, conv, iters
 
     def decode_host(self, syndromes: np.ndarray, out=None):
