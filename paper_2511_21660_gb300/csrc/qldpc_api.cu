@@ -620,9 +620,12 @@ int launch_persistent(const qldpc_decoder *d, const uint64_t *syn, int64_t B, De
     if (!tail) return QLDPC_OK;
     // With a split launch, up to split_clusters records go to it (a cluster of blocks each, all
     // resident) and more to the one-block launch: gross code at p = 0.02, 17 records 30.1 ms
-    // with one block a shot, 24.0 split; 42 31.6 / 28.3; about 130 39 / 69.  A small batch, which
-    // cannot have many, leaves the one-block launch out.
-    const bool one_block = !d->fk_split || B > 8LL * d->split_clusters;
+    // with one block a shot, 24.0 split; 42 31.6 / 28.3; about 130 39 / 69.  The records are
+    // counted on the device, and any number of a batch's shots may have one (syndromes that no
+    // fault set explains), so only a batch of at most split_clusters shots, which cannot pass
+    // that line, leaves the one-block launch out (150 unsolvable gross syndromes, 60 legs: split
+    // alone 14.2 ms, with both queued 6.8; 300: 24.1 / 12.6).
+    const bool one_block = !d->fk_split || B > d->split_clusters;
     if (d->fk_split)
         QL_CUDA(d->fk_split->launch(d->split_clusters, d->split_smem, st, d->split, d->prm, syn, out,
                                     d->counter + 2, map, d->tail,

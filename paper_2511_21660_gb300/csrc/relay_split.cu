@@ -110,7 +110,8 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(NT, MINB)
     const int tid = threadIdx.x, lane = tid & 31;
     const int me = (int)(blockIdx.x % kSplit), cluster = (int)(blockIdx.x / kSplit);
     const int n = (int)min(*tc.count, (unsigned int)tc.cap);
-    // the whole cluster, as are all of them when one block a shot is faster (see setup_split)
+    // the whole cluster, as are all of them when one block a shot is faster (see
+    // launch_persistent)
     if (cluster >= n || n > most) return;
 
     // this block's rows as a graph of their own, for the check pass
