@@ -483,27 +483,38 @@ __device__ __forceinline__ void check_pass(const FusedGraph &g, __half *msg, con
 // -0).  Messages are stored unclamped (the check pass takes their magnitudes' minimum
 // with C); the marginal is clamped.
 //
-// Faults of degree 2 and 3 with their slots in a packed record.
-template <typename MT, int FAULTS>
-__device__ __forceinline__ float fault_update(unsigned char *msg, const Packed<MT, FAULTS> &s,
-                                              float lam, float C) {
+// Faults of degree 2 and 3, by the byte offsets of their slots.
+template <typename MT>
+__device__ __forceinline__ float fault_update(unsigned char *msg, uint32_t o0, uint32_t o1,
+                                              uint32_t o2, bool three, float lam, float C) {
     using R = Raw<MT>;
-    const typename R::T m0 = ld_raw<MT>(msg, s.o0), m1 = ld_raw<MT>(msg, s.o1);
+    const typename R::T m0 = ld_raw<MT>(msg, o0), m1 = ld_raw<MT>(msg, o1);
     typename R::T m2 = 0;
-    if (s.three) m2 = ld_raw<MT>(msg, s.o2);
+    if (three) m2 = ld_raw<MT>(msg, o2);
     const float p1 = R::add(lam, m0), p2 = R::add(p1, m1);
-    Msg<MT>::st(msg, s.o0, R::add(R::add(lam, m1), m2));
-    Msg<MT>::st(msg, s.o1, R::add(p1, m2));
-    if (s.three) Msg<MT>::st(msg, s.o2, p2);
+    Msg<MT>::st(msg, o0, R::add(R::add(lam, m1), m2));
+    Msg<MT>::st(msg, o1, R::add(p1, m2));
+    if (three) Msg<MT>::st(msg, o2, p2);
     const float L = R::add(p2, m2);
     return sizeof(MT) == 4 ? clamp_nan(L, C) : clampc(L, C);
 }
+template <typename MT, int FAULTS>
+__device__ __forceinline__ float fault_update(unsigned char *msg, const Packed<MT, FAULTS> &s,
+                                              float lam, float C) {
+    return fault_update<MT>(msg, s.o0, s.o1, s.o2, s.three, lam, C);
+}
 
-// Any degree up to DV.
+// Any degree up to DV.  Where that is 8, degrees 2 and 3 keep their own code here too: the loop
+// below takes 36 additions whatever the degree, and graphs with more than 64 KB of messages and up
+// to 3072 faults have no packed records (16-slot rows, 1500 checks, 2400 faults of degree 3, 6000
+// shots: 0.70 -> 0.64 ms; 32-slot rows, 600 checks, 2900 faults: 10.6 -> 9.2).  For 4 slots the
+// branch costs a warp of mixed degrees more than it saves (degrees 3 and 4: 0.40 -> 0.43 ms).
 template <typename MT, int DV>
 __device__ __forceinline__ float fault_update(unsigned char *msg, const int (&sl)[DV], int deg,
                                               float lam, float C) {
     using R = Raw<MT>;
+    if (DV > 4 && (deg == 2 || deg == 3))
+        return fault_update<MT>(msg, sl[0], sl[1], sl[2], deg == 3, lam, C);
     typename R::T mu[DV];
 #pragma unroll
     for (int k = 0; k < DV; ++k) {
