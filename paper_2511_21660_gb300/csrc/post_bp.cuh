@@ -61,7 +61,7 @@ __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C,
             if (j < g.N) {
                 int sl[DV];
                 const int deg = load_slots<DV>(g, j, sl);
-                Lam[r] = fault_update<float, DV>(msg, sl, deg, wr[r], C);
+                Lam[r] = fault_update<float, DV>(msg, sl, deg, fs.records, wr[r], C);
             }
         };
         each_fault<VPT>(fs.n, fast, any);

@@ -154,10 +154,12 @@ template <typename MT, int NT, int VPT, bool KEEP = false>
 struct FaultSlots {
     using P = Packed<MT, NT * VPT>;
     int n;
+    bool records;  // the graph has packed records
     uint2 kept[KEEP ? VPT : 1];
     __device__ __forceinline__ void init(const FusedGraph &g) {
         n = 0;
-        if (!P::table(g)) return;
+        records = P::table(g) != nullptr;
+        if (!records) return;
         const int groups = (g.N + 31) >> 5;
         int r = 0;
 #pragma unroll 1
@@ -504,16 +506,17 @@ __device__ __forceinline__ float fault_update(unsigned char *msg, const Packed<M
     return fault_update<MT>(msg, s.o0, s.o1, s.o2, s.three, lam, C);
 }
 
-// Any degree up to DV.  Where that is 8, degrees 2 and 3 keep their own code here too: the loop
-// below takes 36 additions whatever the degree, and graphs with more than 64 KB of messages and up
-// to 3072 faults have no packed records (16-slot rows, 1500 checks, 2400 faults of degree 3, 6000
-// shots: 0.70 -> 0.64 ms; 32-slot rows, 600 checks, 2900 faults: 10.6 -> 9.2).  For 4 slots the
-// branch costs a warp of mixed degrees more than it saves (degrees 3 and 4: 0.40 -> 0.43 ms).
+// Any degree up to DV.  Where that is 8, degrees 2 and 3 of a graph without packed records (more
+// than 64 KB of messages, up to 3072 faults) have their own code here too: the loop below takes 36
+// additions whatever the degree (16-slot rows, 1500 checks, 2400 faults of degree 3, 6000 shots:
+// 0.70 -> 0.64 ms; 32-slot rows, 600 checks, 2900 faults: 10.6 -> 9.2).  With records, what comes
+// here are warps of mixed degrees, which the branch would only split (16-slot rows, degrees 3 to
+// 5: 0.60 -> 0.64 ms; 8-slot rows, degrees 3 and 4: 0.26 -> 0.31).
 template <typename MT, int DV>
 __device__ __forceinline__ float fault_update(unsigned char *msg, const int (&sl)[DV], int deg,
-                                              float lam, float C) {
+                                              bool records, float lam, float C) {
     using R = Raw<MT>;
-    if (DV > 4 && (deg == 2 || deg == 3))
+    if (DV > 4 && !records && (deg == 2 || deg == 3))
         return fault_update<MT>(msg, sl[0], sl[1], sl[2], deg == 3, lam, C);
     typename R::T mu[DV];
 #pragma unroll
@@ -573,7 +576,7 @@ __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned cha
             const float lam = __fadd_rn(bb[r], __fmul_rn(gg[r], Lam[r]));
             int sl[DV];
             const int deg = load_slots<DV>(g, j, sl);
-            L = fault_update<MT, DV>(msg, sl, deg, lam, C);
+            L = fault_update<MT, DV>(msg, sl, deg, fs.records, lam, C);
             Lam[r] = L;
         }
         decide(L);

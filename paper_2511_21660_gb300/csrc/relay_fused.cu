@@ -263,6 +263,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_decode_multi(MultiTable tab,
     int cur = -1;
     FaultSlots<MT, NT, VPT> fs;
     fs.n = 0;
+    fs.records = false;
     RowBits rb;
     rb.part = 0u;
 
