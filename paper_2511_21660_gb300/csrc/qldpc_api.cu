@@ -208,6 +208,36 @@ cudaError_t allow_smem(const void *fn, size_t smem) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+// The library's shape is the narrowest that holds the faults.  Two kinds of graph take another:
+//   * messages above 64 KB, no record in bytes: the first shape that reads records in messages
+//     (6000 shots, 512 x 6 or 256 x 12 -> 640 x 5: 8-slot rows, 2500 checks, 3000 faults 0.68 ->
+//     0.46 ms; 16-slot rows, 1500 checks, 3000 faults 1.16 -> 0.96);
+//   * so many rows that shared memory holds at most 3/5 of the blocks the shape is laid out for:
+//     the wide shape, which needs fewer shots for as many threads (5000 shots, narrow / wide: 1800
+//     faults, 2200 checks, 3 blocks of 5, 16.4 / 10.2 ms; 4000, 3600, 1 of 3 66.5 / 43.4; 8000,
+//     5400, 1 of 2 169 / 88; with 2 of 3 or 3 of 4 the narrow one is as fast or faster: 2400,
+//     1800 16.5 / 17.0, 3500, 2600 33.4 / 38.3).
+int setup_fit(qldpc_decoder *d, bool rec_fits, bool rec8_fits) {
+    auto bytes = [](const FusedKernel &k) { return k.threads * k.vpt <= kByteRecordFaults; };
+    const bool no_records = bytes(*d->fk) && !rec8_fits && rec_fits;
+    if (!no_records && 5 * d->blocks_per_sm > 3 * d->fk->min_blocks) return QLDPC_OK;
+    for (int q = 0; q < d->ntable; ++q) {
+        const FusedKernel &k = d->table[q];
+        if (!holds(k, d->M, d->N)) continue;
+        if (no_records ? bytes(k) : !(k.latency && k.threads > d->fk->threads)) continue;
+        int bps = 0;
+        QL_CUDA(allow_smem(k.decode_fn, d->smem));
+        QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k.decode_fn, k.threads,
+                                                              d->smem));
+        if (bps >= 1) {
+            d->fk = &k;
+            d->blocks_per_sm = bps;
+        }
+        break;
+    }
+    return QLDPC_OK;
+}
+
 // Small batches: with fewer shots than about twice the blocks that a wider shape keeps
 // resident, a shot's latency counts and the narrow shape's full residency does not.
 // Measured (us a launch, narrow / wide): gross code 100 shots 39.5 / 34.3, 608 101 / 87, 2400
@@ -498,6 +528,10 @@ int setup_fused(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_idx
                                                           d->fk->threads, d->smem));
     if (d->blocks_per_sm < 1)
         return fail(QLDPC_ERR_UNSUPPORTED, "the decode kernel cannot be resident on an SM");
+    if (block_threads == 0) {
+        rc = setup_fit(d, rec_fits, rec8_fits);
+        if (rc) return rc;
+    }
     if (d->fk_trace) {
         d->trace_smem = d->smem;
         QL_CUDA(allow_smem(d->fk_trace->trace_fn, d->smem));

@@ -113,6 +113,10 @@ struct TailCont {
 };
 
 // One compiled instance of the fused kernel.
+// Shapes of up to this many faults read the packed slot records in bytes (FusedGraph::var_rec8),
+// larger ones in messages (var_rec).
+constexpr int kByteRecordFaults = 3072;
+
 struct FusedKernel {
     int msg_fp16;   // 0 float32 storage, 1 binary16 storage
     int threads;    // NT

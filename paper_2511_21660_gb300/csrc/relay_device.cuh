@@ -132,7 +132,7 @@ __device__ __forceinline__ int swz(int i) {
 // beside its messages, where the 16-byte table of offsets hit in half the reads.
 template <typename MT, int FAULTS>
 struct Packed {
-    static constexpr bool kBytes = FAULTS <= 3072;
+    static constexpr bool kBytes = FAULTS <= kByteRecordFaults;
     static __device__ __forceinline__ const uint2 *table(const FusedGraph &g) {
         return kBytes ? g.var_rec8 : g.var_rec;
     }
