@@ -78,8 +78,12 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : (VPT <= 8 && DC <= 16 ? 2 
     __shared__ uint32_t s_x[32], s_lk[32], s_sw[32];
     const int tid = threadIdx.x, lane = tid & 31;
 
+    FaultSlots<float, NT, VPT> fs;
+    fs.init(g);
+    const uint32_t part = part_rows<float, NT, DC>(g);
+
     for (;;) {
-        // per-shot registers, declared here so that nothing of them lives across shots
+        // per-shot registers, declared here so that nothing else lives across shots
         float Lam[VPT];
 #pragma unroll
         for (int r = 0; r < VPT; ++r) Lam[r] = 0.0f;
@@ -96,7 +100,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 5 : (VPT <= 8 && DC <= 16 ? 2 
             s_rows = 0;
         }
         plain_bp_marginals<NT, VPT, DC, DV>(g, p.clip, o.bp_iters, syn + (size_t)shot * g.syn_words,
-                                            msg, sg, par, Lam);
+                                            msg, sg, par, fs, part, Lam);
 
         // 2. ranking: candidates Lambda_j < llr_conf, keys (Lambda_j, j)
 #pragma unroll
@@ -241,7 +245,8 @@ OsdKernel osd_entry() {
 }  // namespace
 
 void osd_table(const OsdKernel **out, int *n) {
-    // per (DC, DV) family of the fused layout: the first entry with threads * vpt >= N
+    // per (DC, DV) family of the fused layout: the first entry with threads * vpt >= N that finds
+    // its slot records in the graph
     static const OsdKernel table[] = {
         osd_entry<256, 12, 8, 4>(), osd_entry<512, 8, 8, 4>(),  osd_entry<512, 16, 8, 4>(),
         osd_entry<512, 8, 16, 8>(), osd_entry<512, 16, 16, 8>(),

@@ -160,8 +160,12 @@ int qldpc_osd_create(qldpc_osd **out, int32_t M, int32_t N, const int32_t *row_p
     const OsdKernel *tab = nullptr;
     int ntab = 0;
     osd_table(&tab, &ntab);
+    // a shape of up to kByteRecordFaults faults reads slot records in bytes, which a graph with
+    // more than 64 KB of messages does not have (3000 shots of 2500 checks, 3000 faults: 256 x 12
+    // on the general path 2.23 ms, 512 x 8 with records in messages 1.22)
     for (int q = 0; q < ntab && !o->k; ++q)
-        if (tab[q].dc == DC && tab[q].dv == DV && (long long)tab[q].threads * tab[q].vpt >= N)
+        if (tab[q].dc == DC && tab[q].dv == DV && (long long)tab[q].threads * tab[q].vpt >= N &&
+            (d->fg.var_rec8 || !d->fg.var_rec || tab[q].threads * tab[q].vpt > kByteRecordFaults))
             o->k = &tab[q];
     auto bail = [&](int code) {
         std::string msg = last_error();

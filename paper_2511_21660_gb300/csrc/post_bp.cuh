@@ -19,18 +19,19 @@ namespace {
 // Lam[r]).  Shared memory: the float32 message slots (msg), the staged syndrome (sg) and
 // one parity buffer (par, set by each check pass and otherwise unused).  Re-stages the
 // padding slots first (callers reuse the message area between shots).  Called by every
-// thread of the block; ends with a barrier.
+// thread of the block; ends with a barrier.  fs and part (the thread's rows with padding) are the
+// graph's, set up once a block: 25 iterations of a tiny graph are short against them.
 template <int NT, int VPT, int DC, int DV>
 __device__ __forceinline__ void plain_bp_marginals(const FusedGraph &g, float C, int iters,
                                                    const uint64_t *sy, unsigned char *msg,
                                                    uint32_t *sg, uint32_t *par,
-                                                   float (&Lam)[VPT]) {
+                                                   const FaultSlots<float, NT, VPT> &fs,
+                                                   uint32_t part, float (&Lam)[VPT]) {
     load_syndrome<NT>(g, sy, sg);
     const uint2 *rec = Packed<float, NT * VPT>::table(g) + threadIdx.x;
-    FaultSlots<float, NT, VPT> fs;
-    fs.init(g);
+    pad_rows<float, NT, DC>(g, msg, C);
     RowBits rb;
-    rb.part = setup_rows<float, NT, DC>(g, msg, C);
+    rb.part = part;
     // nu(0) = lambda(0) = w on every edge, Lambda(0) = w
     float wr[VPT];
 #pragma unroll

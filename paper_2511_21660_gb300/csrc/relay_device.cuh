@@ -328,11 +328,9 @@ struct RowBits {
     uint32_t s0, s1, part;
 };
 
-// The rows of the thread that have padding slots; those slots get C, which the check pass
-// keeps there for good.  (Rows past the last check are never visited.)
+// Padding slots get C, which the check pass keeps there for good.
 template <typename MT, int NT, int DC>
-__device__ __forceinline__ uint32_t setup_rows(const FusedGraph &g, unsigned char *msg, float C) {
-    uint32_t m = 0u;
+__device__ __forceinline__ void pad_rows(const FusedGraph &g, unsigned char *msg, float C) {
     const bool half = sizeof(MT) == 2;
     for (int i = threadIdx.x; i < g.Mp; i += NT) {
         const int deg = g.chk_deg[i];
@@ -343,6 +341,13 @@ __device__ __forceinline__ uint32_t setup_rows(const FusedGraph &g, unsigned cha
             Msg<MT>::st(msg, off, C);
         }
     }
+}
+
+// The rows of the thread that have padding slots.  (Rows past the last check are never visited.)
+template <typename MT, int NT, int DC>
+__device__ __forceinline__ uint32_t part_rows(const FusedGraph &g) {
+    uint32_t m = 0u;
+    const bool half = sizeof(MT) == 2;
     const int rows = half ? (g.M + 1) >> 1 : g.M;
     for (int i = threadIdx.x, k = 0; i < rows; i += NT, ++k) {
         const bool full = half ? g.chk_deg[2 * i] == DC && g.chk_deg[2 * i + 1] == DC
@@ -350,6 +355,12 @@ __device__ __forceinline__ uint32_t setup_rows(const FusedGraph &g, unsigned cha
         m |= (full ? 0u : 1u) << k;
     }
     return m;
+}
+
+template <typename MT, int NT, int DC>
+__device__ __forceinline__ uint32_t setup_rows(const FusedGraph &g, unsigned char *msg, float C) {
+    pad_rows<MT, NT, DC>(g, msg, C);
+    return part_rows<MT, NT, DC>(g);
 }
 
 // The syndrome bits of the thread's rows, from the shot's packed words in global memory.
