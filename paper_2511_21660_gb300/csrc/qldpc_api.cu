@@ -224,7 +224,7 @@ int setup_fit(qldpc_decoder *d, bool rec_fits, bool rec8_fits) {
     for (int q = 0; q < d->ntable; ++q) {
         const FusedKernel &k = d->table[q];
         if (!holds(k, d->M, d->N)) continue;
-        if (no_records ? bytes(k) : !(k.latency && k.threads > d->fk->threads)) continue;
+        if (no_records ? bytes(k) : !(k.waves && k.threads > d->fk->threads)) continue;
         int bps = 0;
         QL_CUDA(allow_smem(k.decode_fn, d->smem));
         QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k.decode_fn, k.threads,
@@ -238,18 +238,23 @@ int setup_fit(qldpc_decoder *d, bool rec_fits, bool rec8_fits) {
     return QLDPC_OK;
 }
 
-// Small batches: with fewer shots than about twice the blocks that a wider shape keeps
-// resident, a shot's latency counts and the narrow shape's full residency does not.
-// Measured (us a launch, narrow / wide): gross code 100 shots 39.5 / 34.3, 608 101 / 87, 2400
-// 145 / 165; 720 faults 608 39 / 31, 2400 56 / 67; 8064 faults 304 112 / 101, 1200 283 / 288;
-// 72 faults 2400 141 / 107.
+// Small batches: a call ends with its longest shots, and a narrow block runs a shot's iterations
+// slower than a wide one; up to a number of shots per resident wide block (FusedKernel::waves) that
+// outweighs the narrow shape's throughput.  Measured (narrow / wide): gross code 100 shots 39.5 /
+// 34.3 us, 608 101 / 87, 2400 145 / 165; 8064 faults 304 112 / 101, 1200 283 / 288: 2 shots a block.
+// Graphs of up to 1024 faults have the longest tails against their launch: 720 faults 5000 shots
+// 186 / 164 us, 10000 237 / 233; 144 faults (code capacity) 600 388 / 274, 5000 469 / 395, 10000
+// 547 / 579; 400 faults and checks 5000 1.54 / 1.07 ms: 12 shots a block.  72 to 96 faults 32 x 3
+// against 64 x 4: 80 faults, 60 checks 5000 575 / 463 us, 20000 607 / 574, 72 faults 10000 171 /
+// 191: 3 shots a block.  Blocks of 512 threads and more are wide themselves (3168 faults, 307 shots:
+// 640 x 5 53 us, 1024 x 8 77).
 int setup_small(qldpc_decoder *d) {
+    if (d->fk->threads >= 512) return QLDPC_OK;
     for (int q = 0; q < d->ntable && !d->fk_small; ++q)
-        if (d->table[q].latency && holds(d->table[q], d->M, d->N)) d->fk_small = &d->table[q];
-    if (!d->fk_small || d->fk_small->threads <= d->fk->threads) {
-        d->fk_small = nullptr;
-        return QLDPC_OK;
-    }
+        if (d->table[q].waves && d->table[q].threads > d->fk->threads &&
+            holds(d->table[q], d->M, d->N))
+            d->fk_small = &d->table[q];
+    if (!d->fk_small) return QLDPC_OK;
     int bps = 0;
     QL_CUDA(allow_smem(d->fk_small->decode_fn, d->smem));
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, d->fk_small->decode_fn,
@@ -259,7 +264,7 @@ int setup_small(qldpc_decoder *d) {
         return QLDPC_OK;
     }
     d->small_grid = d->num_sms * bps;
-    d->small_max = 2LL * d->small_grid;
+    d->small_max = (int64_t)d->fk_small->waves * d->small_grid;
     return QLDPC_OK;
 }
 
@@ -932,9 +937,13 @@ int qldpc_decode_batch_multi(qldpc_decoder *const *decoders, int32_t n_codes,
         if (ptrs[q] && !is_device_ptr(ptrs[q]))
             return fail(QLDPC_ERR_INVALID_ARG, "argument %d is not device memory", q);
     // one shape serves every code: the largest code's wide one (small codes leave most of a
-    // narrow block's fault slots empty), or the first that holds every code
+    // narrow block's fault slots empty: 8064 faults with 2736 and 720, 256 x 32 52.4, 1024 x 8 40.5
+    // ms), its own where that has few slots a thread (72 and 144 faults, 20000 shots: 64 x 4 0.18,
+    // 256 x 4 0.35 ms; 2736 and 3168: 640 x 5 1.72, 1024 x 8 3.04), or the first that holds every
+    // code
     const qldpc_decoder *db = decoders[big];
-    const FusedKernel *fk = db->fk_small ? db->fk_small : db->fk;
+    const FusedKernel *fk = db->fk;
+    if (db->fk_small && (B <= db->small_max || fk->vpt > 6)) fk = db->fk_small;
     auto holds_all = [&](const FusedKernel &k) {
         for (int c = 0; c < n_codes; ++c)
             if (!holds(k, decoders[c]->M, decoders[c]->N)) return false;

@@ -122,7 +122,7 @@ struct FusedKernel {
     int threads;    // NT
     int min_blocks; // launch-bounds residency target
     int vpt;        // faults per thread (register-resident)
-    bool latency;   // a shape for batches too small to fill the SMs with narrow blocks
+    int waves;      // > 0: a shape for small batches, of up to so many shots per resident block
     int dc, dv;     // max check / fault degree supported
     const void *decode_fn;   // __global__ symbol of the decode kernel
     cudaError_t (*launch_decode)(dim3 grid, size_t smem, cudaStream_t st, const FusedGraph &g,

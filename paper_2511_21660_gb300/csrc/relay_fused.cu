@@ -413,12 +413,10 @@ using MsgT = __half;
 using MsgT = float;
 #endif
 
-constexpr bool kLatency = QL_DC == 8;
-
-template <int NT, int VPT, int MINB, bool TRACE, bool LATENCY = false>
+template <int NT, int VPT, int MINB, bool TRACE, int WAVES = 0>
 FusedKernel entry() {
     FusedKernel k;
-    k.latency = LATENCY;
+    k.waves = QL_DC == 8 ? WAVES : 0;
     k.msg_fp16 = QL_MSG_F16;
     k.threads = NT;
     k.min_blocks = MINB;
@@ -460,7 +458,7 @@ void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
     // (threads, faults per thread, min resident blocks): the first entry that holds the graph
     // (threads * vpt >= N) is used unless the caller asks for a block size; the last
     // entry also serves the trace kernel; the 1024-thread entries serve the resuming
-    // launch of the tail continuation; the entries marked kLatency serve small batches.
+    // launch of the tail continuation; the entries with a number of waves serve small batches.
     //
     // Rows of up to 8 slots: the blocks are narrow, with as many faults per thread as the
     // registers hold at full residency, since the cost of an iteration that does not depend
@@ -473,13 +471,13 @@ void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
     static const FusedKernel table[] = {
 #if QL_DC == 8
         entry<32, 3, 32, false>(),
-        entry<64, 4, 16, false, kLatency>(),
+        entry<64, 4, 16, false, 3>(),
         entry<64, 8, 16, false>(),
         entry<64, 12, 16, false>(),
         entry<64, 13, 12, false>(),
         entry<128, 8, 8, false>(),
 #endif
-        entry<256, 4, 4, false, kLatency>(),
+        entry<256, 4, 4, false, 12>(),
 #if QL_DC == 8
         entry<128, 10, 6, false>(),
         entry<128, 12, 6, false>(),
@@ -489,7 +487,7 @@ void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
         entry<256, 11, 4, false>(),
         entry<256, 12, 4, false>(),
 #endif
-        entry<512, 6, 2, false, kLatency>(),
+        entry<512, 6, 2, false, 2>(),
         entry<256, 12, 4, false>(),
         entry<384, 8, 3, false>(),
         entry<640, 5, 2, false>(),
@@ -504,7 +502,7 @@ void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
         entry<384, 18, 2, false>(),
         entry<256, 32, 2, false>(),
 #endif
-        entry<1024, 8, 1, false, kLatency>(),
+        entry<1024, 8, 1, false, 2>(),
         entry<512, 16, 1, false>(),
         entry<512, 32, 1, true>(),
     };
