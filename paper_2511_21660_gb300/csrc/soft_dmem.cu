@@ -25,10 +25,15 @@ namespace qldpc {
 namespace {
 
 // Threads per block of the forward: float32 rows of up to 8 edges run 4 blocks of 320 (48
-// registers; 2048 gross shots 0.91 ms, 384 0.92, 512 0.95); wider rows and FP64, whose rows take
-// longer, keep wide blocks (rows of up to 32, 64 shots: 512 0.33 ms, 320 0.40).
+// registers; 2048 gross shots 0.91 ms, 384 0.92, 512 0.95) where the state leaves room for 5 (the
+// SM's shared memory is then not what bounds the residency).  Larger graphs keep wide blocks, which
+// make up in threads for the blocks that do not fit (320 / 512: 1216 shots of 3600 faults, 4 blocks,
+// 0.636 / 0.625 ms, one shot 0.217 / 0.176; 5760, 3 blocks, 1.28 / 1.07; 8064, one block, 2.70 /
+// 2.01), and so do wider rows and FP64, whose rows take longer (rows of up to 32, 64 shots: 512 0.33
+// ms, 320 0.40).
+constexpr int kFwdWide = 512;
 template <typename T, int DCM>
-constexpr int kFwdThreads = sizeof(T) == 4 && DCM == 8 ? 320 : 512;
+constexpr int kFwdMany = sizeof(T) == 4 && DCM == 8 ? 320 : kFwdWide;
 // Threads per block of the adjoint, and its resident blocks per SM (float32 rows of up to 8
 // edges; its register budget follows from them).
 #ifndef SOFT_BWD_THREADS
@@ -344,9 +349,8 @@ __device__ __forceinline__ void copy_state(const T *src, T *dst, int n) {
 
 // Forward.  Shared memory: nu[E], Lam[N] (a.sst values).  The state before iterations
 // 1, K + 1, 2K + 1, ... is stored as a checkpoint.
-template <typename T, int DCM>
-__global__ void __launch_bounds__(kFwdThreads<T, DCM>) soft_forward(SoftArgs<T> a) {
-    constexpr int NT = kFwdThreads<T, DCM>;
+template <typename T, int DCM, int NT>
+__global__ void __launch_bounds__(NT) soft_forward(SoftArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SoftGraph &g = a.g;
     T *nu = reinterpret_cast<T *>(smem_raw);
@@ -573,6 +577,26 @@ size_t bwd_smem(const SoftGraph &g, int Tit) {
     return sizeof(T) * ((size_t)soft_state_values(g) + Tit);
 }
 
+template <typename T, int DCM, int NT>
+cudaError_t launch_forward(const SoftArgs<T> &a, size_t sm, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(soft_forward<T, DCM, NT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    soft_forward<T, DCM, NT><<<a.B, NT, sm, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Whether five blocks with `sm` bytes of dynamic shared memory fit an SM (1 KB a block is the
+// system's, and the block's own arrays take less than 256 bytes).
+cudaError_t five_fit(size_t sm, bool *yes) {
+    int device = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
+    *yes = e == cudaSuccess && 5 * (sm + 1024 + 256) <= (size_t)per_sm;
+    return e;
+}
+
 template <typename T, int DCM>
 cudaError_t run_forward_t(const SoftLaunch &L, cudaStream_t st) {
     SoftArgs<T> a{};
@@ -595,11 +619,11 @@ cudaError_t run_forward_t(const SoftLaunch &L, cudaStream_t st) {
     a.marg = static_cast<T *>(L.marg);
     a.sst = soft_state_values(L.g);
     const size_t sm = fwd_smem<T>(L.g);
-    cudaError_t e = cudaFuncSetAttribute(soft_forward<T, DCM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    soft_forward<T, DCM><<<L.B, kFwdThreads<T, DCM>, sm, st>>>(a);
-    e = cudaGetLastError();
+    bool many = false;
+    cudaError_t e = five_fit(sm, &many);
+    if (e == cudaSuccess)
+        e = many ? launch_forward<T, DCM, kFwdMany<T, DCM>>(a, sm, st)
+                 : launch_forward<T, DCM, kFwdWide>(a, sm, st);
     if (e != cudaSuccess) return e;
     const T scale = T(1) / ((T)L.B * (T)L.g.N);
     return sum_shots<T>(a.shot_loss, L.B, 1, scale, nullptr, static_cast<T *>(L.loss), st);
