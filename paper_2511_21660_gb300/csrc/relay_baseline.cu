@@ -15,7 +15,8 @@ namespace {
 constexpr int BASE_THREADS = 256;
 constexpr unsigned FULL = 0xffffffffu;
 
-__device__ __forceinline__ float clampc(float x, float c) { return fminf(fmaxf(x, -c), c); }
+// Keeps a NaN, as the oracle's comparisons do.
+__device__ __forceinline__ float clampc(float x, float c) { return x > c ? c : (x < -c ? -c : x); }
 
 struct BaseSmem {
     float *nu, *mu, *Lam, *lam0, *lam;

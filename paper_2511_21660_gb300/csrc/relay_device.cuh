@@ -35,10 +35,11 @@ struct Msg<__half> {
     }
 };
 
-__device__ __forceinline__ float clampc(float x, float c) { return fminf(fmaxf(x, -c), c); }
-
-// The clamp that keeps a NaN (clampc turns it into -c).
-__device__ __forceinline__ float clamp_nan(float x, float c) {
+// Clamp to [-c, c] that keeps a NaN, as the oracle's comparisons do (fminf and fmaxf would turn it
+// into -c).  Memory strengths beyond about 1e8 can overflow the two terms of lambda to opposite
+// infinities; such a fault is not decided, and its messages neither bound a minimum nor turn a sign
+// (a NaN from arithmetic has sign bit 0).
+__device__ __forceinline__ float clampc(float x, float c) {
     float y;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(x), "f"(-c));
     asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(y), "f"(c));
@@ -509,7 +510,7 @@ __device__ __forceinline__ float fault_update(unsigned char *msg, uint32_t o0, u
     Msg<MT>::st(msg, o1, R::add(p1, m2));
     if (three) Msg<MT>::st(msg, o2, p2);
     const float L = R::add(p2, m2);
-    return sizeof(MT) == 4 ? clamp_nan(L, C) : clampc(L, C);
+    return clampc(L, C);
 }
 template <typename MT, int FAULTS>
 __device__ __forceinline__ float fault_update(unsigned char *msg, const Packed<MT, FAULTS> &s,

@@ -243,7 +243,7 @@ __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(NT, MINB)
                         Peer<MT>::st(at[v][k] == zero ? trash : at[v][k], x);
                         s = R::add(s, mu[v][k]);
                     }
-                    Lam[v] = sizeof(MT) == 4 ? clamp_nan(s, C) : clampc(s, C);
+                    Lam[v] = clampc(s, C);
                     const uint32_t d = __float_as_uint(Lam[v]) >> 31;
                     dm |= d << v;
 #pragma unroll
