@@ -12,6 +12,7 @@
 #include "qldpc.h"
 #include "qldpc_internal.h"
 #include "relay_split.h"
+#include "smem_limit.h"
 
 namespace qldpc {
 

@@ -199,15 +199,6 @@ bool holds(const FusedKernel &k, int M, int N) {
     return (long long)k.threads * k.vpt >= N && 32LL * k.threads >= rows;
 }
 
-// Raises a kernel's limit of dynamic shared memory to `smem` (the limit belongs to the kernel,
-// which handles of several graphs share: it is never lowered).
-cudaError_t allow_smem(const void *fn, size_t smem) {
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, fn);
-    if (e != cudaSuccess || (size_t)a.maxDynamicSharedSizeBytes >= smem) return e;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 // The library's shape is the narrowest that holds the faults.  Two kinds of graph take another:
 //   * messages above 64 KB, no record in bytes: the first shape that reads records in messages
 //     (6000 shots, 512 x 6 or 256 x 12 -> 640 x 5: 8-slot rows, 2500 checks, 3000 faults 0.68 ->
