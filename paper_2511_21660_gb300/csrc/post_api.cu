@@ -52,7 +52,7 @@ cudaError_t configure_kernel(const void *fn, int threads, size_t smem, int devic
     cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     *fits = e == cudaSuccess && smem <= (size_t)optin;
     if (e != cudaSuccess || !*fits) return e;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(fn, smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, threads, smem);
     *fits = e == cudaSuccess && bps >= 1;
     *grid = num_sms * std::max(bps, 1);

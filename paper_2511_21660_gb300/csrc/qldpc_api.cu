@@ -593,8 +593,7 @@ int setup_baseline(qldpc_decoder *d, const int32_t *row_ptr, const int32_t *col_
     if (d->smem > (size_t)optin)
         return fail(QLDPC_ERR_UNSUPPORTED, "baseline kernel needs %zu B of shared memory, above %d",
                     d->smem, optin);
-    QL_CUDA(cudaFuncSetAttribute(baseline_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)d->smem));
+    QL_CUDA(allow_smem(baseline_fn(), d->smem));
     QL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->blocks_per_sm, baseline_fn(), 256,
                                                           d->smem));
     d->block_threads = 256;

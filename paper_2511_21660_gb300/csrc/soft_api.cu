@@ -164,6 +164,8 @@ int qldpc_soft_create(qldpc_soft **out, int32_t M, int32_t N, const int32_t *row
     if (soft_smem_backward(g, s->T, s->fp64) > (size_t)optin)
         return cleanup(fail(QLDPC_ERR_UNSUPPORTED, "soft state needs %zu B of shared memory, above %d",
                             soft_smem_backward(g, s->T, s->fp64), optin));
+    e = soft_allow_smem(g, s->dc_max, s->T, s->fp64);
+    if (e != cudaSuccess) return cleanup(fail(QLDPC_ERR_CUDA, "%s", cudaGetErrorString(e)));
     // one 8-byte record per fault (its first three slots and its degree) replaces the two
     // dependent reads of var_ptr and var_edges in the kernels' fault loops
     const bool rec = pad && slots < 65536;

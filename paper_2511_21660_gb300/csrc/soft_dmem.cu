@@ -19,6 +19,7 @@
 // Lambda(T)); in the others the recompute forms only the tanh rows of that iteration's
 // input.  Per-shot gradients are summed over shots in a fixed order, so results are
 // deterministic.
+#include "smem_limit.h"
 #include "soft_internal.h"
 
 namespace qldpc {
@@ -579,9 +580,6 @@ size_t bwd_smem(const SoftGraph &g, int Tit) {
 
 template <typename T, int DCM, int NT>
 cudaError_t launch_forward(const SoftArgs<T> &a, size_t sm, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(soft_forward<T, DCM, NT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     soft_forward<T, DCM, NT><<<a.B, NT, sm, st>>>(a);
     return cudaGetLastError();
 }
@@ -595,6 +593,19 @@ cudaError_t five_fit(size_t sm, bool *yes) {
         e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
     *yes = e == cudaSuccess && 5 * (sm + 1024 + 256) <= (size_t)per_sm;
     return e;
+}
+
+// Shared memory of a handle's launches (set when it is created).
+template <typename T, int DCM>
+cudaError_t allow_t(const SoftGraph &g, int T_it) {
+    bool many = false;
+    cudaError_t e = five_fit(fwd_smem<T>(g), &many);
+    if (e != cudaSuccess) return e;
+    e = allow_smem(many ? (const void *)soft_forward<T, DCM, kFwdMany<T, DCM>>
+                        : (const void *)soft_forward<T, DCM, kFwdWide>,
+                   fwd_smem<T>(g));
+    if (e != cudaSuccess) return e;
+    return allow_smem((const void *)soft_backward<T, DCM>, bwd_smem<T>(g, T_it));
 }
 
 template <typename T, int DCM>
@@ -651,11 +662,8 @@ cudaError_t run_backward_t(const SoftLaunch &L, cudaStream_t st) {
     a.shot_adj = static_cast<T *>(L.shot_adj);
     a.sst = soft_state_values(L.g);
     const size_t sm = bwd_smem<T>(L.g, L.T_it);
-    cudaError_t e = cudaFuncSetAttribute(soft_backward<T, DCM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     soft_backward<T, DCM><<<L.B, SOFT_BWD_THREADS, sm, st>>>(a);
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const T scale = T(1) / ((T)L.B * (T)L.g.N);
     const T *up = static_cast<const T *>(L.upstream);
@@ -671,6 +679,11 @@ size_t soft_smem_forward(const SoftGraph &g, int fp64) {
 }
 size_t soft_smem_backward(const SoftGraph &g, int T_it, int fp64) {
     return fp64 ? bwd_smem<double>(g, T_it) : bwd_smem<float>(g, T_it);
+}
+
+cudaError_t soft_allow_smem(const SoftGraph &g, int dc_max, int T_it, int fp64) {
+    if (fp64) return dc_max <= 8 ? allow_t<double, 8>(g, T_it) : allow_t<double, 32>(g, T_it);
+    return dc_max <= 8 ? allow_t<float, 8>(g, T_it) : allow_t<float, 32>(g, T_it);
 }
 
 cudaError_t soft_run_forward(const SoftLaunch &L, cudaStream_t st) {

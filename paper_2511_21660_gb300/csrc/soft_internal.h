@@ -37,6 +37,8 @@ inline int soft_state_values(const SoftGraph &g) { return (g.E + g.N + 3) & ~3; 
 
 size_t soft_smem_forward(const SoftGraph &g, int fp64);
 size_t soft_smem_backward(const SoftGraph &g, int T_it, int fp64);
+// Raises the limits of dynamic shared memory of the kernels that a handle launches.
+cudaError_t soft_allow_smem(const SoftGraph &g, int dc_max, int T_it, int fp64);
 cudaError_t soft_run_forward(const SoftLaunch &L, cudaStream_t st);
 cudaError_t soft_run_backward(const SoftLaunch &L, cudaStream_t st);
 
