@@ -604,7 +604,7 @@ def mixed_batch_variant(args, dev, stream, flush):
                                device=dev.index)
         except Exception:
             continue
-        if big.info.block_threads != bt:
+        if bt and big.info.block_threads != bt:  # 0: the library's own choice
             big.close()
             continue
         decs = [RelayDecoder(P.row_ptr, P.col_idx, P.p, g, cfg, device=dev.index)

@@ -19,7 +19,10 @@ import numpy as np
 
 from .qldpc import QldpcError, RelayConfig, RelayDecoder
 
-CANDIDATES = (32, 64, 128, 256, 384, 512, 640, 768, 1024)
+# 0: the library's choice, which also has a shape of its own for small batches; an explicit size
+# runs one shape for batches of every size
+CANDIDATES = (0, 32, 64, 128, 256, 384, 512, 640, 768, 1024)
+TIE = 1.02               # the library's choice is kept within this factor of the fastest
 TAIL_OPTIONS = (0, -1)   # the library default (continuation after T_1 + 8 T_r), off
 CACHE = os.path.join(os.path.expanduser("~"), ".cache", "qldpc", "tuning.json")
 
@@ -46,11 +49,23 @@ def _sample_digest(syndromes) -> str:
     return f"B{s.shape[0]}:{int(torch.sum(s.to(torch.float64) * 1e-9).item() * 1e6)}"
 
 
+def pick(timings: dict) -> tuple:
+    """(block_threads, tail_cut_iters) of {"bt/tail": ms}: the fastest, or the library's own choice
+    (block size 0) when that is as fast: on the sample it often is the very shape that an
+    explicit size names, and it keeps its small-batch shape."""
+    best = min(timings, key=timings.get)
+    own = {k: v for k, v in timings.items() if k.startswith("0/")}
+    if own and min(own.values()) <= TIE * timings[best]:
+        best = min(own, key=own.get)
+    return tuple(int(x) for x in best.split("/"))
+
+
 def tune(row_ptr, col_idx, priors, gamma_table, config: RelayConfig, syndromes,
          repeats: int = 3, cache: str | None = CACHE, block_sizes=CANDIDATES,
          tail_options=TAIL_OPTIONS):
     """Time every compiled block size with each tail setting on `syndromes` (int64 CUDA
-    tensor [B, words]).  Returns ((block_threads, tail_cut_iters), {"bt/tail": ms}).
+    tensor [B, words]).  Returns ((block_threads, tail_cut_iters), {"bt/tail": ms}); pick says
+    which.
     Shapes the graph does not fit are skipped (block size 0: the library's choice); the
     answer is cached per key."""
     import torch
@@ -88,8 +103,7 @@ def tune(row_ptr, col_idx, priors, gamma_table, config: RelayConfig, syndromes,
             dec.close()
     if not timings:
         raise RuntimeError("no compiled block shape fits this problem")
-    best_key = min(timings, key=timings.get)
-    best = tuple(int(x) for x in best_key.split("/"))
+    best = pick(timings)
     if cache:
         try:
             os.makedirs(os.path.dirname(cache), exist_ok=True)
