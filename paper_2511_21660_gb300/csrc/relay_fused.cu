@@ -488,7 +488,9 @@ void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
         entry<256, 12, 4, false>(),
 #endif
         entry<512, 6, 2, false, 2>(),
+#if QL_DC != 8
         entry<256, 12, 4, false>(),
+#endif
         entry<384, 8, 3, false>(),
         entry<640, 5, 2, false>(),
         entry<768, 4, 2, false>(),
