@@ -542,7 +542,7 @@ __device__ __forceinline__ float fault_update(unsigned char *msg, const int (&sl
         float v = p;
 #pragma unroll
         for (int k2 = k + 1; k2 < DV; ++k2) v = R::add(v, mu[k2]);
-        if (k < deg) Msg<MT>::st(msg, sl[k], clampc(v, C));
+        if (k < deg) Msg<MT>::st(msg, sl[k], v);
         p = R::add(p, mu[k]);
     }
     return clampc(p, C);
