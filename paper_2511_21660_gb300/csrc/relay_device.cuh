@@ -184,10 +184,11 @@ struct FaultSlots {
 // The per-fault loops: fast(r) for the packed slots and any(r) for the others.  (One loop body
 // with a branch per fault on its degree, a ballot and a bitmap store took 50 instructions a
 // warp of faults, this form 31; gross code, 30,000 shots: 2.50 -> 1.96 ms with the leg
-// start's same change.)  The shapes
-// are chosen so that a graph fills every fault slot but the last, and then the loop runs
-// without a branch between faults, which lets their loads overlap; on other graphs it
-// branches once per group of faults (and takes any(r) in the group where the packed slots end).
+// start's same change.)  Where a warp's packed slots are all or all but the last (the detector
+// models whose fault count fills their shape, as 6 to 13 rounds of the bivariate-bicycle codes do
+// but for a few sizes) the loop runs without a branch between faults, which lets their loads
+// overlap.  Otherwise it branches once per group of four, and takes any(r) for the whole group
+// where the packed slots end (up to three packed slots a thread on the general path).
 template <int VPT, typename Fast, typename Any>
 __device__ __forceinline__ void each_fault(int packed, Fast fast, Any any) {
     if (packed >= VPT - 1) {

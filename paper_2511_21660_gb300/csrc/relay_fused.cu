@@ -463,11 +463,13 @@ void QL_EXPAND(QL_P, QL_DC, QL_DV)(const FusedKernel **out, int *n) {
     // Rows of up to 8 slots: the blocks are narrow, with as many faults per thread as the
     // registers hold at full residency, since the cost of an iteration that does not depend
     // on the faults (barriers, the convergence test, the check pass's uneven rows) is per
-    // warp.  Each entry's reach is chosen so that the graphs it is used for fill all fault
-    // slots but the last (each_fault).  Measured, old shape -> this one: 72 faults 256 x 4 ->
-    // 32 x 3 2.26 -> 0.59 ms (60,000 shots), 720 faults 256 x 4 -> 64 x 12 1.13 -> 0.75 ms,
-    // gross code 512 x 6 -> 256 x 11 1.88 -> 1.59 ms (30,000), 8064 faults 1024 x 8 -> 256 x
-    // 32 1.72 -> 1.49 ms (8,000).
+    // warp.  The reaches are chosen so that the detector models of the three codes fill all
+    // fault slots but the last at most of their usual numbers of rounds (each_fault; counted, no
+    // warp does for the 72-qubit code at 2, 3, 5, 9, 14, 15 and 18 rounds, the 144-qubit code at 0,
+    // 1, 2, 7 and 16, the 288-qubit code at 0, 3, 4, 11, 13, 16 and 17).  Measured, old shape ->
+    // this one: 72 faults 256 x 4 -> 32 x 3 2.26 -> 0.59 ms (60,000 shots), 720 faults 256 x 4 ->
+    // 64 x 12 1.13 -> 0.75 ms, gross code 512 x 6 -> 256 x 11 1.88 -> 1.59 ms (30,000), 8064 faults
+    // 1024 x 8 -> 256 x 32 1.72 -> 1.49 ms (8,000).
     static const FusedKernel table[] = {
 #if QL_DC == 8
         entry<32, 3, 32, false>(),
