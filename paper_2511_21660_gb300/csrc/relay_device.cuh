@@ -525,7 +525,10 @@ __device__ __forceinline__ float fault_update(unsigned char *msg, const Packed<M
 // 0.70 -> 0.64 ms; 32-slot rows, 600 checks, 2900 faults: 10.6 -> 9.2).  With records, what comes
 // here are warps of mixed degrees, which the branch would only split (16-slot rows, degrees 3 to
 // 5: 0.60 -> 0.64 ms; 8-slot rows, degrees 3 and 4: 0.26 -> 0.31).
-template <typename MT, int DV>
+// CUT: values above C are cut to it before the store.  The check pass bounds them anyway; the decode
+// kernels of the 8-slot float32 family do it because without this instruction the compiler spills 8
+// bytes in the iteration loop of the 256 x 11 shape (10^5 gross shots 4.68 -> 4.74 ms).
+template <typename MT, int DV, bool CUT = false>
 __device__ __forceinline__ float fault_update(unsigned char *msg, const int (&sl)[DV], int deg,
                                               bool records, float lam, float C) {
     using R = Raw<MT>;
@@ -543,6 +546,7 @@ __device__ __forceinline__ float fault_update(unsigned char *msg, const int (&sl
         float v = p;
 #pragma unroll
         for (int k2 = k + 1; k2 < DV; ++k2) v = R::add(v, mu[k2]);
+        if (CUT) asm("min.NaN.f32 %0, %1, %2;" : "=f"(v) : "f"(v), "f"(C));
         if (k < deg) Msg<MT>::st(msg, sl[k], v);
         p = R::add(p, mu[k]);
     }
@@ -564,7 +568,7 @@ __device__ __forceinline__ int check_of_slot(int off) {
 // The decision of a fault is the sign bit of its marginal (never -0, see fault_update), shifted
 // into a mask; the bitmap words and the parity flips follow for the warps that decided any.
 // Returns the thread's decided faults (bit VPT-1-r: fault threadIdx.x + r*NT has F_j = 1).
-template <typename MT, int NT, int VPT, int DC, int DV, typename FS>
+template <typename MT, int NT, int VPT, int DC, int DV, bool CUT = false, typename FS>
 __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned char *msg, uint32_t *fw,
                                            uint32_t *par, const FS &fs, float (&Lam)[VPT],
                                            const float (&bb)[VPT], const float (&gg)[VPT],
@@ -589,7 +593,7 @@ __device__ __forceinline__ uint32_t fault_pass(const FusedGraph &g, unsigned cha
             const float lam = __fadd_rn(bb[r], __fmul_rn(gg[r], Lam[r]));
             int sl[DV];
             const int deg = load_slots<DV>(g, j, sl);
-            L = fault_update<MT, DV>(msg, sl, deg, fs.records, lam, C);
+            L = fault_update<MT, DV, CUT>(msg, sl, deg, fs.records, lam, C);
             Lam[r] = L;
         }
         decide(L);

@@ -54,6 +54,7 @@ struct ShotState {
 // records kept 1.15 ms).
 template <int NT, int VPT, int MINB>
 constexpr bool kKeep = QL_DC == 8 && (65536 / (NT * MINB) / 8 * 8) >= 5 * VPT + 31;
+constexpr bool kCut = QL_DC == 8 && !QL_MSG_F16;  // see fault_update
 constexpr long long kNoWeight = 0x7fffffffffffffffLL;
 
 // Relay on one shot: the leg schedule around the check and fault passes.  Per
@@ -153,7 +154,7 @@ __device__ __forceinline__ void decode_shot(const FusedGraph &g, const DevParams
         do {
             check_pass<NT, DC>(g, reinterpret_cast<MT *>(msg), sg, pc, rb, C);
             __syncthreads();
-            dm = fault_pass<MT, NT, VPT, DC, DV>(g, msg, fw, pc, fs, Lam, bb, gg, C);
+            dm = fault_pass<MT, NT, VPT, DC, DV, kCut>(g, msg, fw, pc, fs, Lam, bb, gg, C);
             __syncthreads();
             ++t;
             conv = warp_converged(pc, g.m_words);
